@@ -403,11 +403,13 @@ int bs_debug_eigh_banded(int n, int bw, const double *A, int nval, double *w, do
  * of 16 bytes or more per basis state); 11..20 = the core-grouped path for
  * FP32 with k = 4 or 8: a persistent kernel computes the pn term per
  * (Z-1)-proton core (up to four destination rows per staged source row) into
- * Z partial vectors (11, 13, 15, 16: 18 consumer warps with one 32-column
+ * Z partial vectors (11, 13, 15: 18 consumer warps with one 32-column
  * slice each; 12, 14: 9 warps with two slices each, a long and a short list;
- * 15, 16: as 13 with the whole 227 KB of shared memory and three or four
+ * 15: as 13 with the whole 227 KB of shared memory and three
  * neutron-list buffers; 17, 18, 19: 227 KB, two list buffers; 20: 227 KB,
- * three list buffers); in 11, 12, 17
+ * three list buffers; 16: the pn term by pairs of a (Z-1)-proton and an
+ * (N-1)-neutron core, a dense product per group of neutron cores, for every
+ * k and for W-truncated bases too); in 11, 12, 17
  * the pipelined kernel computes the like-particle terms into one more (17:
  * the first pipelined variant that fits, for neutron sectors wider than 576
  * columns); in 13..16 and 18..20 a second persistent kernel computes the pp
@@ -415,14 +417,17 @@ int bs_debug_eigh_banded(int n, int bw, const double *A, int nval, double *w, do
  * (Z-2)-proton core into C(Z,2) more and a row-tile kernel (4 rows per CTA,
  * 2 in 19 and 20, column tiles of 576 for wider sectors; 18: the first pipelined
  * variant that fits) the nn term and the proton single-particle energies
- * into one more; a last kernel
+ * into one more (16 with k = 1, 2 or a W-truncated basis: panels of x in
+ * shared memory for both like-particle terms, which add the partial vectors);
+ * a last kernel
  * sums the partial vectors in a fixed order (workspace: up to
  * (Z + C(Z,2) + 1) x dim x k floats, allocated on first use, or by
  * bs_lanczos before it captures a graph; a first call inside a stream
- * capture without it falls back to the pipelined kernel).  A mode that does not fit
+ * capture without it falls back to another kernel).  A mode that does not fit
  * the basis falls back to the tiled kernel.  0 (default) = the mode bs_autotune picked
- * for the call's (k, dtype), else mode 13 where it applies (FP32, k = 4, 8),
- * else the first pipelined variant, else the first row variant.  All modes give the same result up to summation order.
+ * for the call's (k, dtype), else for FP32 one by the size of the basis (16
+ * or 20 for large ones, where they apply), else the first pipelined variant,
+ * else the first row variant.  All modes give the same result up to summation order.
  * Errors: BS_EINVAL. */
 int bs_set_kernel(bs_ctx *ctx, int mode);
 
@@ -469,7 +474,8 @@ int bs_kernel_times(bs_ctx *ctx, float *ms, int *n);
  * ("pp_ptr", "pp_src", "pp_coef", "nn_*", "p1_ptr", "p1_ent", "p1_cls",
  * "n1_*", "wpn", "links", "ops", "op_lists", "stats", the pipelined and
  * core-grouped kernels' tables "pe_*", "ww", "ww_off", "core_units",
- * "core_src", "wc", "pp_units", "pps_row", "pps_w", "pdiag") into `out` (HOST,
+ * "core_src", "wc", "pp_units", "pps_row", "pps_w", "pdiag", the pair-core
+ * kernel's "pr_*") into `out` (HOST,
  * caller-allocated; NULL to query the size).  *nbytes receives the size in
  * bytes.  Works on host-only contexts (bs_create with cuda_device = -1),
  * so the host builders can be checked on a machine without a GPU.

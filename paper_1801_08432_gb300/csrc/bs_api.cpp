@@ -290,6 +290,51 @@ int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std
         (R == 2 ? D.nnntasks2 : D.nnntasks4) = (int)nt.size();
         if ((rc = put(D, dst, nt.data(), nt.size(), err))) return rc;
     }
+    for (int spc = 0; spc < 2; ++spc) {   // like-particle panels
+        Device::LikeDev &q = D.like[spc];
+        LikePanels O;
+        build_like_panels(B, spc, 8, O);
+        q.max_n = O.max_n;
+        q.pw = like_panel_width(O.max_n);
+        if (!q.pw) continue;
+        LikeLists L;
+        build_like_lists(B, spc, spc ? T.nn : T.pp, spc ? T.nnx : T.ppx, L);
+        if ((rc = put(D, q.ptr, L.ptr.data(), L.ptr.size(), err))) return rc;
+        if ((rc = put(D, q.ent, L.ent.data(), L.ent.size(), err))) return rc;
+        if ((rc = put(D, q.pieces, O.pieces.data(), O.pieces.size(), err))) return rc;
+        for (int v = 0; v < 4; ++v) {
+            build_like_panels(B, spc, q.pw >> v, O);
+            q.npanels[v] = (int)O.panels.size();
+            if ((rc = put(D, q.panels[v], O.panels.data(), O.panels.size(), err))) return rc;
+        }
+    }
+    if (T.pair.on) {   // pair-core pn kernel
+        const PairTables &R = T.pair;
+        D.pr_ncn = R.ncn;
+        if ((rc = put(D, D.pr_colpos, R.colpos.data(), R.colpos.size(), err))) return rc;
+        if ((rc = put(D, D.pr_nsign, R.nsign.data(), R.nsign.size(), err))) return rc;
+        f = cast<float>(R.w);
+        if ((rc = put(D, D.pr_w, f.data(), f.size(), err))) return rc;
+        if ((rc = put(D, D.pr_recs, R.recs.data(), R.recs.size(), err))) return rc;
+        for (int v = 0; v < 3; ++v) {
+            const int cap = pair_cap_cols(4 >> v, R.max_rec);
+            if (v > 0 && D.pr[v - 1].nitems && D.pr[v - 1].cols >= R.max_cols) { D.pr[v] = D.pr[v - 1]; continue; }
+            PairItems O;
+            // a proton core's rows all at once, or this many components are not taken together: every
+            // part of its rows would gather all of x again
+            if (cap < R.max_cols || !build_pair_items(R, cap, O)) continue;
+            Device::PairDev &q = D.pr[v];
+            q.nitems = (int)O.items.size();
+            q.cols = O.max_cols;
+            q.max_tiles = O.max_tiles;
+            q.max_rows = O.max_rows;
+            q.max_rec = O.max_rec;
+            if ((rc = put(D, q.items, O.items.data(), O.items.size(), err))) return rc;
+            if ((rc = put(D, q.tiles, O.tiles.data(), O.tiles.size(), err))) return rc;
+            if ((rc = put(D, q.rows, O.rows.data(), O.rows.size(), err))) return rc;
+            if ((rc = put(D, q.store, O.store.data(), O.store.size(), err))) return rc;
+        }
+    }
     f = cast<float>(T.ww);
     if ((rc = put(D, D.ww32, f.data(), f.size(), err))) return rc;
     return BS_OK;
@@ -431,7 +476,7 @@ int bs_load_interaction(bs_ctx *c, const double *spe, int n_spe, const bs_tbme *
         rc = build_tables(c->basis, c->inter, c->tab, c->err, nsm);
         if (rc) return rc;
         if (c->device >= 0) {
-            if (c->adj_gpp) { cudaFree(c->adj_gpp); cudaFree(c->adj_gnn); cudaFree(c->adj_rho); }
+                if (c->adj_gpp) { cudaFree(c->adj_gpp); cudaFree(c->adj_gnn); cudaFree(c->adj_rho); }
             c->adj_gpp = c->adj_gnn = c->adj_rho = nullptr;
             rc = upload(c->basis, c->inter, c->tab, c->dev, c->err);
             if (rc) { release(c->dev); return rc; }
@@ -837,7 +882,27 @@ int bs_debug_table(bs_ctx *c, const char *name, void *out, int64_t *nbytes)
         else if (s == "pps_row") use(T.pps_row.data(), T.pps_row.size() * 4);
         else if (s == "pps_w") use(T.pps_w.data(), T.pps_w.size() * 8);
         else if (s == "pdiag") use(T.pdiag.data(), T.pdiag.size() * 8);
-        else if (s == "n1e_base") {
+        else if (s == "pr_colpos") use(T.pair.colpos.data(), T.pair.colpos.size() * 2);
+        else if (s == "pr_nsign") use(T.pair.nsign.data(), T.pair.nsign.size() * 4);
+        else if (s == "pr_w") use(T.pair.w.data(), T.pair.w.size() * 8);
+        else if (s == "pr_recs") use(T.pair.recs.data(), T.pair.recs.size() * sizeof(PairRec));
+        else if (s.size() > 3 && s.substr(0, 3) == "pr_" && (s.back() == '1' || s.back() == '2' || s.back() == '4')) {
+            // items for 1, 2 or 4 components at a time: "pr_items4", "pr_tiles4", "pr_rows4", "pr_store4", ...
+            PairItems O;
+            const int cap = pair_cap_cols(s.back() - '0', T.pair.max_rec);
+            if (T.pair.on) build_pair_items(T.pair, cap, O);
+            auto raw = [&](const void *p, size_t b) {
+                tmp.assign((b + 7) / 8, 0);
+                if (b) std::memcpy(tmp.data(), p, b);
+                use(tmp.data(), b);
+            };
+            s.pop_back();
+            if (s == "pr_items") raw(O.items.data(), O.items.size() * sizeof(PairItem));
+            else if (s == "pr_tiles") raw(O.tiles.data(), O.tiles.size() * sizeof(PairTile));
+            else if (s == "pr_rows") raw(O.rows.data(), O.rows.size() * sizeof(PairRec));
+            else if (s == "pr_store") raw(O.store.data(), O.store.size() * sizeof(PairRow));
+            else { c->err = "unknown table"; return BS_EINVAL; }
+        } else if (s == "n1e_base") {
             for (size_t k = 0; k < T.n1e_col.size(); ++k) { tmp.push_back(T.n1e_col[k]); tmp.push_back(T.n1e_slice[k]); }
             use(tmp.data(), tmp.size() * 8);
         } else if (s == "nne_base") {

@@ -206,6 +206,9 @@ cudaError_t launch_hx_pipe(const bs_ctx *c, const void *x, void *y, int k, bs_dt
 cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dtype dt, cudaStream_t s, int v,
                            bool &used, cudaEvent_t t0, cudaEvent_t t1);
 
+// modes of bs_set_kernel the default rule names
+constexpr int kPairMode = 16, kCoreMode = 20;
+
 static int kslot(int k)
 {
     return k == 1 ? 0 : k == 2 ? 1 : k == 4 ? 2 : 3;
@@ -213,9 +216,9 @@ static int kslot(int k)
 
 // Kernel choice: mode 1 = tiled kernel; mode 2 + v = row kernel variant v;
 // mode 2 + R + v = pipelined kernel variant v (R = number of row variants);
-// mode 0 = the variant the autotuner picked for (k, dtype), else the first
-// pipelined variant, else the first row variant.  A row or pipelined variant
-// that does not fit the basis falls back to the tiled kernel.
+// then the core-grouped modes; mode 0 = the mode the autotuner picked for
+// (k, dtype), else one chosen by the size of the basis.  A variant that does
+// not fit the basis falls back to the tiled kernel.
 int launch_hx(const bs_ctx *c, const void *x, void *y, int k, bs_dtype dt, void *stream, std::string &err)
 {
     cudaStream_t s = (cudaStream_t)stream;
@@ -231,12 +234,37 @@ int launch_hx(const bs_ctx *c, const void *x, void *y, int k, bs_dtype dt, void 
     const int R = row_variants();
     if (mode == 0) mode = c->tuned[dt == BS_F64 ? 0 : 1][kslot(k)];
     if (mode == 0 && e == cudaSuccess) {
-        // not tuned: the core-grouped path where it applies, else the first
-        // pipelined variant, else the first row variant
-        e = launch_hx_core(c, x, y, k, dt, s, 2, used, t0, t1);
-        core_used = used;
-        if (e == cudaSuccess && !used) e = launch_hx_pipe(c, x, y, k, dt, s, 0, used);
-        if (!used) mode = 2;
+        const int64_t dim = c->basis.dim;
+        if (dt == BS_F64 || c->dev.trunc) {
+            // the first pipelined variant, else the first row variant, else the tiled kernel
+            e = launch_hx_pipe(c, x, y, k, dt, s, 0, used);
+            if (!used) mode = 2;
+        } else {
+            // FP32, not tuned.  Measured on this chip, us per product of k = 4 (k = 2) by the tiled / pipelined
+            // (row) / core-grouped / pair-core kernels:
+            //   sd 4p4n 58 / 51 / 82 / 67 (47 / 71 / - / 56);  pf 3p3n 203 / 152 / 168 / 163 (161 / 179 / - / 109);
+            //   pf 4p3n 571 / 741 / 929 / 685 (449 / 762 / - / 353);  pf 4p4n 2847 / 2103 / 1232 / 1141 (2138 / 2236 / - / 725);
+            //   pf 6p2n (neutron sectors of 30) 985 / 5779 / 9782 / - (772 / 4947 / - / -);
+            // at k = 8 the core-grouped kernels lead from 100,000 states and sectors of 64 columns on.
+            const int nN = c->dev.max_nN;
+            const bool small = dim < 100000, narrow = nN < 64;
+            if (!small && narrow) mode = 1;                            // the wide kernels give a thread a column
+            else if (k < 4) mode = small ? 2 : kPairMode;
+            else if (small) mode = 2 + R;                              // one CTA per row fills the chip
+            else if (k == 4 && nN < 256) mode = dim < 300000 ? 2 + R : 1;
+            else mode = k == 4 ? kPairMode : kCoreMode;
+            if (mode == kPairMode || mode == kCoreMode) {
+                // a form that does not fit this basis: the next one
+                for (int m : {mode, (int)kCoreMode, 13})
+                    if (e == cudaSuccess && !used) e = launch_hx_core(c, x, y, k, dt, s, m - 2 - R - pipe_variants(), used, t0, t1);
+                core_used = used;
+                if (!used) mode = 2 + R;
+            }
+            if (e == cudaSuccess && !used && mode == 2 + R) {
+                e = launch_hx_pipe(c, x, y, k, dt, s, 0, used);
+                if (!used) mode = 2;
+            }
+        }
     }
     const int P = pipe_variants();
     if (e == cudaSuccess && !used && mode >= 2 + R + P) {

@@ -34,6 +34,8 @@ namespace bs {
 
 using namespace tma;
 
+cudaError_t launch_hx_pair(const bs_ctx *c, const float *x, float *part, int k, cudaStream_t s, bool &used);
+cudaError_t launch_hx_like(const bs_ctx *c, const float *x, float *y, int k, cudaStream_t s, const float *part, int nz);
 cudaError_t launch_hx_pipe_combine(const bs_ctx *c, const void *x, void *y, int k, bs_dtype dt, cudaStream_t s, int v,
                                    const void *part, int nz, bool skip_pp, bool &used);
 
@@ -869,6 +871,7 @@ struct CoreVariant {
     bool pp;         // pp term by (Z-2)-proton cores, nn by row tiles of nn_rows rows
     int nn_rows;
     int nlb;         // neutron-list buffers (0: three if the ring keeps seven slots, else two)
+    bool pair;       // the pn term by pairs of cores (bs_hx_pair.cu) instead
 };
 
 // Modes 11.. in this order.  The last two spend the whole 227 KB on three or
@@ -882,7 +885,7 @@ struct CoreVariant {
 // 2-row tiles with the three list buffers of mode 15.
 constexpr CoreVariant kCoreVariants[] = {{18, 1, 200 * 1024, false, 0, 0}, {9, 2, 200 * 1024, false, 0, 0},
                                          {18, 1, 200 * 1024, true, 4, 0},  {9, 2, 200 * 1024, true, 4, 0},
-                                         {18, 1, 227 * 1024, true, 4, 3},  {18, 1, 227 * 1024, true, 4, 4},
+                                         {18, 1, 227 * 1024, true, 4, 3},  {18, 1, 227 * 1024, true, 2, 2, true},
                                          {18, 1, 227 * 1024, false, 0, 2}, {18, 1, 227 * 1024, true, 0, 2},
                                          {18, 1, 227 * 1024, true, 2, 2},  {18, 1, 227 * 1024, true, 2, 3}};
 constexpr int kNumCore = 10;
@@ -995,6 +998,19 @@ size_t part_bytes(const bs_ctx *c, int k)
     return (size_t)(c->dev.nz + c->dev.nzpp + 1) * (size_t)c->basis.dim * (size_t)k * sizeof(float);
 }
 
+size_t pair_bytes(const bs_ctx *c, int k)
+{
+    return (size_t)c->basis.Z * (size_t)c->basis.dim * (size_t)k * sizeof(float);
+}
+
+// The pair-core kernel without the core-grouped like-particle kernels: its Z
+// partial vectors go to the like-particle panels.
+bool pair_applies(const bs_ctx *c, int k, bs_dtype dt)
+{
+    bool fits = false;
+    return dt == BS_F32 && like_applies(c) && launch_hx_pair(c, nullptr, nullptr, k, nullptr, fits) == cudaSuccess && fits;
+}
+
 bool core_applies(const bs_ctx *c, int k, bs_dtype dt)
 {
     return !c->dev.trunc && dt == BS_F32 && (k == 4 || k == 8) && c->dev.ncunits > 0 && c->dev.nz > 0;
@@ -1006,8 +1022,7 @@ int core_variants() { return kNumCore; }
 
 int prepare_hx(const bs_ctx *c, int k, bs_dtype dt, std::string &err)
 {
-    if (!core_applies(c, k, dt)) return BS_OK;
-    const size_t need = part_bytes(c, k);
+    const size_t need = core_applies(c, k, dt) ? part_bytes(c, k) : pair_applies(c, k, dt) ? pair_bytes(c, k) : 0;
     if (c->core_part_bytes >= need) return BS_OK;
     if (c->core_part) cudaFree(c->core_part);
     c->core_part = nullptr;
@@ -1030,13 +1045,22 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
                            bool &used, cudaEvent_t t0, cudaEvent_t t1)
 {
     used = false;
-    if (!core_applies(c, k, dt) || v < 0 || v >= kNumCore) return cudaSuccess;
-    if (c->core_part_bytes < part_bytes(c, k)) {
+    if (v < 0 || v >= kNumCore) return cudaSuccess;
+    const bool pair = kCoreVariants[v].pair, core = core_applies(c, k, dt);
+    if (!(core && !pair) && !(pair && pair_applies(c, k, dt))) return cudaSuccess;
+    if (c->core_part_bytes < (core ? part_bytes(c, k) : pair_bytes(c, k))) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         cudaError_t e = cudaStreamIsCapturing(s, &cap);
         if (e != cudaSuccess) return e;
         std::string err;
         if (cap != cudaStreamCaptureStatusNone || prepare_hx(c, k, dt, err) != BS_OK) return cudaSuccess;
+    }
+    if (!core) {
+        cudaError_t e;
+        if (t0 && (e = cudaEventRecord(t0, s)) != cudaSuccess) return e;
+        if ((e = launch_hx_pair(c, (const float *)x, (float *)c->core_part, k, s, used)) != cudaSuccess) return e;
+        if (t1 && (e = cudaEventRecord(t1, s)) != cudaSuccess) return e;
+        return launch_hx_like(c, (const float *)x, (float *)y, k, s, (const float *)c->core_part, c->basis.Z);
     }
     const bool pp = kCoreVariants[v].pp;
     const int R = kCoreVariants[v].nn_rows;
@@ -1058,7 +1082,8 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
     // node in a captured graph), before the timed window of the dominant kernel
     if (c->dev.core_next && (e = cudaMemsetAsync(c->dev.core_next, 0, 2 * sizeof(int), s)) != cudaSuccess) return e;
     if (t0 && (e = cudaEventRecord(t0, s)) != cudaSuccess) return e;
-    e = k == 8 ? launch_core_k<8>(c, xf, part, s, v, used) : launch_core_k<4>(c, xf, part, s, v, used);
+    if (pair) e = launch_hx_pair(c, xf, part, k, s, used);
+    else e = k == 8 ? launch_core_k<8>(c, xf, part, s, v, used) : launch_core_k<4>(c, xf, part, s, v, used);
     if (e != cudaSuccess || !used) return e;
     if (t1 && (e = cudaEventRecord(t1, s)) != cudaSuccess) return e;
     int nz = c->dev.nz;

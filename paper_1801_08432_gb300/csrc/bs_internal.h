@@ -224,7 +224,70 @@ struct PPUnit {
     int64_t doff;
 };
 
+// pn term by pairs of cores (bs_pair.cpp, bs_hx_pair.cu).
+struct PairRec {           // a pair (proton state k, neutron state l) that one proton core and one group of neutron cores leave free
+    uint32_t xoff;         // first basis index of the row cp + k in the block of the group's cn + l
+    uint32_t yoff;         // the same row's first column among the proton core's output columns
+    uint32_t srec;         // 31 - l, and in bit 31 whether the sign of a+_k on cp is -1
+    uint32_t wj;           // place in the key's W matrix | l << 16 | round << 24
+};
+struct PairRow {           // an output row: cp + i in one block
+    int64_t elem;          // first basis index
+    int ycol, n;           // first output column, columns
+    int part;              // partial vector: the rank of i in cp + i
+    int state, sign, pad;  // i; 1: the sign of a+_i on cp is -1
+};
+struct PairGroup { int rec0, nrec, core0, ncore, woff, np; };
+struct PairCore { int rec0, nrec, grp0, ngrp, row0, nrow; };
+constexpr int kPairCores = 128;   // neutron cores of a tile
+constexpr int kPairRows = 16;     // pairs ij of a tile per subset of proton states
+struct PairTile {          // pairs ij (four subsets of proton states) x neutron cores of one group, summed over all its pairs kl
+    int rec0, nrec;        // pairs kl, in the item's records
+    int core0, ncore;
+    int woff, np;          // W matrix of the key, its width
+    uint16_t row0[4];      // pairs ij per subset, in the item's rows, by round
+    uint8_t nrow[4];
+    uint16_t first[4];     // bit r: row r is the first of its round
+    int pad;
+};
+struct PairItem { int rec0, nrec, tile0, ntile, row0, nrow, store0, nstore, cols, pad[3]; };
+struct PairTables {
+    bool on = false;
+    int ncn = 0, max_rec = 0;
+    int64_t max_cols = 0;            // output columns of the proton core with the most
+    std::vector<uint16_t> colpos;    // [states][ncn]: column of cn + s in its neutron sector, 0xFFFF if there is none
+    std::vector<uint32_t> nsign;     // per neutron core: bit s set where the sign of a+_s is -1
+    std::vector<double> w;           // per key: [kl][ij]
+    std::vector<PairRec> recs;
+    std::vector<uint8_t> rec_state;  // proton state of every record (host only)
+    std::vector<PairGroup> grps;
+    std::vector<PairCore> cores;
+    std::vector<PairRow> rows;
+};
+struct PairItems {
+    std::vector<PairItem> items;
+    std::vector<PairTile> tiles;
+    std::vector<PairRec> rows;
+    std::vector<PairRow> store;
+    int max_cols = 0, max_tiles = 0, max_rows = 0, max_rec = 0;
+};
+
+// Like-particle matrices with uniform lists (bs_hx_like.cu).
+struct LikeEnt { int32_t src; float coef; };     // source SD among those of its (2M, parity)
+struct LikeLists {
+    std::vector<int64_t> ptr;                    // per SD of the species
+    std::vector<LikeEnt> ent;
+};
+struct LikePiece { int g0, n; int64_t off; int nN, pad; };   // SDs g0 .. g0 + n - 1 of the panel: one block
+struct LikePanel { int64_t row0; int n, pos0, npos, piece0, npiece, pad; };
+struct LikePanels {
+    std::vector<LikePanel> panels;
+    std::vector<LikePiece> pieces;
+    int max_n = 0;
+};
+
 struct Tables {
+    PairTables pair;
     int grid = 152;                      // CTAs of the persistent core-grouped kernels (units are balanced for it)
     LikeJumps pp, nn;                    // moves inside a sector (diagonal and SPE included)
     LikeCross ppx, nnx;                  // moves between sectors (W-truncated bases only)
@@ -352,6 +415,27 @@ struct Device {
     // neutron like-particle kernel over tiles of R proton rows (R = 2, 4): (block, first row)
     int2 *nntasks2 = nullptr, *nntasks4 = nullptr;
     int nnntasks2 = 0, nnntasks4 = 0;
+    // like-particle matrices: protons, neutrons; panels for k = 1, 2, 4, 8
+    struct LikeDev {
+        int64_t *ptr = nullptr;
+        LikeEnt *ent = nullptr;
+        LikePiece *pieces = nullptr;
+        LikePanel *panels[4] = {nullptr, nullptr, nullptr, nullptr};
+        int npanels[4] = {0, 0, 0, 0}, max_n = 0, pw = 0;
+    } like[2];
+    // pair-core pn kernel: items for 4, 2 and 1 components at a time (shared where the rows of a proton core fit)
+    struct PairDev {
+        PairItem *items = nullptr;
+        PairTile *tiles = nullptr;
+        PairRec *rows = nullptr;
+        PairRow *store = nullptr;
+        int nitems = 0, cols = 0, max_tiles = 0, max_rows = 0, max_rec = 0;
+    } pr[3];
+    uint16_t *pr_colpos = nullptr;
+    uint32_t *pr_nsign = nullptr;
+    float *pr_w = nullptr;
+    PairRec *pr_recs = nullptr;
+    int pr_ncn = 0;
     std::vector<void *> owned;   // every cudaMalloc above
 };
 
@@ -398,6 +482,13 @@ int build_basis(Basis &B, const bs_orbit *orbits, int n_orbits, int Z, int N, in
 int build_interaction(const Basis &B, const double *spe, int n_spe, const bs_tbme *tbme, int n_tbme,
                       Interaction &I, std::string &err);
 int build_tables(const Basis &B, const Interaction &I, Tables &T, std::string &err, int grid = 152);
+void build_like_lists(const Basis &B, int spc, const LikeJumps &L, const LikeCross &X, LikeLists &O);
+void build_like_panels(const Basis &B, int spc, int pos, LikePanels &O);
+int like_panel_width(int max_n);
+bool like_applies(const bs_ctx *ctx);
+void build_pair_tables(const Basis &B, const Interaction &I, PairTables &T, int64_t max_cols);
+bool build_pair_items(const PairTables &T, int cap, PairItems &O);
+int pair_cap_cols(int cp, int max_rec);
 int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std::string &err);
 void release(Device &D);
 int launch_hx(const bs_ctx *ctx, const void *x, void *y, int k, bs_dtype dt, void *stream, std::string &err);

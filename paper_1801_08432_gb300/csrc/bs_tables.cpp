@@ -1237,6 +1237,7 @@ int build_tables(const Basis &B, const Interaction &I, Tables &T, std::string &e
         T.ops_nn += onn;
     }
     T.ops_per_vector = ops;
+    build_pair_tables(B, I, T.pair, pair_cap_cols(1, 0));
     if (B.trunc) return BS_OK;   // the core-grouped tables assume one neutron sector per proton sector
     {   // the pp-core kernel packs a destination row and its partial rank into one int
         const int Z = B.sp[0].nparticles;
