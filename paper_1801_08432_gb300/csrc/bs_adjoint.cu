@@ -4,20 +4,25 @@
 // kernels).  H is linear in theta = (SPEs, TBMEs) through the decoupling of
 // Eq. (hamdef) / Eq. (xpndef), so
 //   d/dtheta_t (gy . H x) = sum over jumps of (dc_jump / dtheta_t) gy[dst] . x[src].
-// The kernels here reduce gy . x over the jumps into transition densities:
-//   pp: one value per pp jump (destination SD row . source SD row),
-//   nn: one value per nn jump (summed over the proton rows of the block),
-//   pn: one value per (proton operator a, neutron operator b) of a W_pn
-//       group, summed over all proton jump x neutron jump pairs using (a, b);
-// the host then splits pp/nn values into two-body moves and contracts
-// everything with dW/dtheta.  Products of FP32 vectors are formed in FP32
-// and summed in FP64; pn densities use FP64 atomics (the order of those
+// The kernels here reduce gy . x over the jumps into two-body transition
+// densities rho(ij,kl), one small matrix per pair key (2m, parity); the host
+// contracts them with dW/dtheta.  Through the cores left by the pair kl (and
+// ij) each is a Gram matrix,
+//   rho(ij,kl) = sum_cores (sign gy[core + ij]) . (sign x[core + kl]),
+// with the cores (Z-1 protons, N-1 neutrons) for pn, (N-2 neutrons, any
+// proton SD) for nn and (Z-2 protons, any neutron SD) for pp: see
+// adj_gram.  Spaces its tables do not cover (more than 32 states per
+// species) take the kernels before it: one value per pp and nn jump, split
+// into two-body moves on the host, and the pn densities by atomics per pair
+// of jumps.  Products of FP32 vectors are formed in FP32; their sums carry
+// 48 bits or more, and are collected with FP64 atomics (the order of those
 // additions, and so the last bits, may differ from run to run).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 
 #include "bs_internal.h"
 
@@ -223,30 +228,470 @@ int launch_adj(bs_ctx *c, const T *x, const T *gy, cudaStream_t s, std::vector<i
     return BS_OK;
 }
 
-// dWpp/dWpn of every TBME as given (unit interactions through the same decoupling)
-int build_derivatives(bs_ctx *c)
-{
-    const int nt = (int)c->tbme_in.size();
-    c->dWpp.assign(nt, {});
-    c->dWpn.assign(nt, {});
-    std::vector<double> zero(c->spe_in.size(), 0.0);
-    for (int t = 0; t < nt; ++t) {
-        bs_tbme one = c->tbme_in[(size_t)t];
-        one.v = 1.0;
-        Interaction U;
-        std::string err;
-        int rc = build_interaction(c->basis, zero.data(), (int)zero.size(), &one, 1, U, err);
-        if (rc) { c->err = err; return rc; }
-        for (size_t i = 0; i < U.Wpp.size(); ++i)
-            if (U.Wpp[i] != 0.0) c->dWpp[(size_t)t].emplace_back((int64_t)i, U.Wpp[i]);
-        for (size_t i = 0; i < U.Wpn.size(); ++i)
-            if (U.Wpn[i] != 0.0) c->dWpn[(size_t)t].emplace_back((int64_t)i, U.Wpn[i]);
+// ---------------------------------------------------------------- Gram matrices
+constexpr int kGramThreads = 256;
+constexpr int kGramTile = 64;          // at most 64 x 64 pairs: 16 x 16 threads of 4 x 4
+
+struct GramArgs {
+    const GramUnit *units;
+    const GramRow *rows;
+    const int *range;                  // units of CTA b: range[b] .. range[b + 1] - 1
+    const uint16_t *colpos;            // neutron cores (bs_pair.cpp)
+    const uint32_t *nsign;
+    int ncn;
+};
+
+// One partial sum: FP64, or double-float for FP32 vectors (the FP32 pipe adds
+// a term to hi + lo in 7 operations; one FP64 add takes as long as 60).
+template <typename T>
+struct GramSum;
+template <>
+struct GramSum<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double f) { v += f; }
+    __device__ __forceinline__ double get() const { return v; }
+};
+template <>
+struct GramSum<float> {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float f)
+    {
+        const float t = hi + f, b = t - hi;
+        lo += (hi - (t - b)) + (f - b);
+        hi = t;
     }
-    c->have_dW = true;
+    __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+};
+
+// rho(ij,kl) += sum over a unit's columns (pn: neutron cores of one group;
+// pp: neutron SDs; nn: proton SDs) of gy[ij] . x[kl].  A CTA stages the two
+// [pairs][columns][K] tiles in shared memory, each element once and with its
+// sign, and every element meets all the pairs of the other tile: 4 x 4
+// pairs per thread, in registers over all of the CTA's consecutive units of
+// one matrix (units are ordered by matrix).  (ceil(np / 4))^2 threads cover a
+// matrix; a small one is covered several times, by slices that take every
+// S-th column.  FP32 add issue bounds it (K multiply-adds and 7 adds per
+// pair and column), against one FP64 shared-memory atomic per pair of jumps
+// before: 48Cr k = 4, 26.7 ms for pn alone.
+template <typename T, int K>
+__global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T *__restrict__ x, const T *__restrict__ gy,
+                                                            double *__restrict__ rho)
+{
+    constexpr int E = K * (int)sizeof(T);                 // bytes of an element
+    constexpr int CH = 256 / E;                           // columns staged at a time
+    constexpr int PAD = E < 16 ? K : 16 / (int)sizeof(T);   // neighbouring pairs' elements lie in other banks
+    constexpr int LD = CH * K + PAD;
+    __shared__ __align__(16) T sx[kGramTile * LD], sg[kGramTile * LD];
+    __shared__ int rowa[kGramTile], rowb[kGramTile];      // record of a tile's pair, -1: not in this unit
+    const int tid = threadIdx.x;
+    GramSum<T> acc[4][4];
+    int out = -1, ga = 1, gb = 1, np = 0, ta = 0, tb = 0;   // the matrix tile the sums belong to
+    int64_t out_at = 0;
+    auto flush = [&]() {
+        if (out < 0) return;
+        const int t = tid % (ga * gb), ia = t % ga, ib = t / ga;
+        if (tid < kGramThreads / (ga * gb) * (ga * gb)) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int a = ia + ga * p, b = ib + gb * q;
+                    const double v = acc[p][q].get();
+                    if (a < ta && b < tb && v != 0.0) atomicAdd(rho + out_at + (int64_t)b * np + a, v);
+                }
+        }
+    };
+    for (int u = A.range[blockIdx.x]; u < A.range[blockIdx.x + 1]; ++u) {
+        const GramUnit U = A.units[u];
+        if (U.tile != out) {
+            flush();
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[p][q] = GramSum<T>();
+            out = U.tile;
+            out_at = U.out;
+            np = U.np;
+            ta = U.ta;
+            tb = U.tb;
+            ga = (ta + 3) / 4;
+            gb = (tb + 3) / 4;
+        }
+        const int nt = ga * gb, S = kGramThreads / nt;
+        const int slice = tid / nt, t = tid % nt, ia = t % ga, ib = t / ga;
+        __syncthreads();   // the last unit's tiles and records are read
+        if (tid < kGramTile) rowa[tid] = rowb[tid] = -1;
+        __syncthreads();
+        for (int r = tid; r < U.na; r += kGramThreads) rowa[A.rows[U.a0 + r].pos - U.pa] = U.a0 + r;
+        for (int r = tid; r < U.nb; r += kGramThreads) rowb[A.rows[U.b0 + r].pos - U.pb] = U.b0 + r;
+        __syncthreads();
+        for (int c0 = 0; c0 < U.ncol; c0 += CH) {
+            if (c0) __syncthreads();
+            for (int n = tid; n < (ta + tb) * CH; n += kGramThreads) {
+                const int slot = n / CH, c = n % CH, col = c0 + c;
+                const bool isx = slot >= ta;
+                const int sl = isx ? slot - ta : slot;
+                const int r = isx ? rowb[sl] : rowa[sl];
+                T *d = (isx ? sx : sg) + sl * LD + c * K;
+                int64_t at = -1;
+                bool neg = false;
+                if (r >= 0 && col < U.ncol) {
+                    const GramRow R = A.rows[r];
+                    neg = R.sign;
+                    if (U.core0 >= 0) {   // pn: the column of core + l, and the sign of a+_l on the core
+                        const int p = __ldg(A.colpos + (size_t)R.l * A.ncn + U.core0 + col);
+                        if (p != 0xFFFF) at = R.off + p;
+                        neg = neg != (bool)(__ldg(A.nsign + U.core0 + col) >> R.l & 1u);
+                    } else {
+                        at = R.off + (int64_t)col * U.stride;
+                    }
+                }
+                T v[K];
+#pragma unroll
+                for (int q = 0; q < K; ++q) v[q] = T(0);
+                if (at >= 0) {
+                    const T *s = (isx ? x : gy) + at * K;
+                    if constexpr (E >= 16) {
+#pragma unroll
+                        for (int q = 0; q < K; q += 16 / (int)sizeof(T))
+                            *reinterpret_cast<int4 *>(v + q) = __ldg(reinterpret_cast<const int4 *>(s + q));
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < K; ++q) v[q] = __ldg(s + q);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < K; ++q) d[q] = neg ? -v[q] : v[q];
+            }
+            __syncthreads();
+            const int cn = min(CH, U.ncol - c0);
+            if (slice < S) {
+                for (int c = slice; c < cn; c += S) {
+                    T a[4][K], b[4][K];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const T *pa = sg + (ia + ga * p) * LD + c * K, *pb = sx + (ib + gb * p) * LD + c * K;
+#pragma unroll
+                        for (int q = 0; q < K; ++q) {
+                            a[p][q] = pa[q];
+                            b[p][q] = pb[q];
+                        }
+                    }
+#pragma unroll
+                    for (int p = 0; p < 4; ++p)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            T f = a[p][0] * b[q][0];
+#pragma unroll
+                            for (int k = 1; k < K; ++k) f = fma(a[p][k], b[q][k], f);
+                            acc[p][q].add(f);
+                        }
+                }
+            }
+        }
+    }
+    flush();
+}
+
+// Overlaps per SD: pd[g] = gy . x over the other species' SDs of proton SD g, one warp each.
+template <typename T, int K>
+__global__ void adj_pdiag(const RowTask *tasks, int n, const DevBlock *blocks, const T *__restrict__ x, const T *__restrict__ gy,
+                          double *__restrict__ pd)
+{
+    const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (w >= n) return;
+    const RowTask t = tasks[w];
+    const DevBlock D = blocks[t.block];
+    const int64_t base = (D.off + (int64_t)t.row * D.nN) * K;
+    double s = 0.0;
+    for (int c = lane; c < D.nN; c += 32) s += dotk<T, K>(gy + base + (int64_t)c * K, x + base + (int64_t)c * K);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) pd[D.p_start + t.row] = s;
+}
+
+// nd[g] likewise for neutron SDs: a CTA takes 128 columns and 32 rows of a block.
+constexpr int kNdRows = 32;
+template <typename T, int K>
+__global__ void adj_ndiag(const int4 *tasks, const DevBlock *blocks, const T *__restrict__ x, const T *__restrict__ gy,
+                          double *__restrict__ nd)
+{
+    const int4 t = tasks[blockIdx.x];   // block, first row, first column
+    const DevBlock D = blocks[t.x];
+    const int c = t.z + (int)threadIdx.x;
+    if (c >= D.nN) return;
+    double s = 0.0;
+    for (int r = t.y; r < min(D.nP, t.y + kNdRows); ++r) {
+        const int64_t at = (D.off + (int64_t)r * D.nN + c) * K;
+        s += dotk<T, K>(gy + at, x + at);
+    }
+    atomicAdd(nd + D.n_start + c, s);
+}
+
+template <typename T, int K>
+cudaError_t launch_gram(bs_ctx *c, const T *x, const T *gy, cudaStream_t s)
+{
+    const AdjPlan &P = c->adj;
+    const Device &D = c->dev;
+    GramArgs A{P.units, P.rows, P.range, P.colpos, P.nsign, P.ncn};
+    if (P.nctas > 0) adj_gram<T, K><<<P.nctas, kGramThreads, 0, s>>>(A, x, gy, P.out);
+    adj_pdiag<T, K><<<(D.nrtasks + 3) / 4, 128, 0, s>>>(D.rtasks, D.nrtasks, D.blocks, x, gy, P.out + P.pd);
+    if (P.nnd > 0) adj_ndiag<T, K><<<P.nnd, 128, 0, s>>>(P.ndtasks, D.blocks, x, gy, P.out + P.nd);
+    return cudaGetLastError();
+}
+
+// (N-2)-cores of one species: for every pair key the pairs each core leaves free, with the SD they lead to.
+struct Core2 {
+    uint64_t bits;
+    std::vector<std::pair<int, int64_t>> at;   // position in the key's pair list, global SD
+    int key;
+};
+
+void core2_lists(const Basis &B, const Interaction &I, int spc, std::vector<Core2> &out)
+{
+    const Species &S = B.sp[spc];
+    const int ns = (int)B.st.size();
+    if (S.nparticles < 2) return;
+    std::vector<uint64_t> cores;
+    for (uint64_t r : S.bits)
+        for (int a = 0; a < ns; ++a)
+            if (r >> a & 1)
+                for (int b = a + 1; b < ns; ++b)
+                    if (r >> b & 1) cores.push_back(r & ~(1ULL << a) & ~(1ULL << b));
+    std::sort(cores.begin(), cores.end());
+    cores.erase(std::unique(cores.begin(), cores.end()), cores.end());
+    for (size_t key = 0; key < I.pairs_by_key.size(); ++key)
+        for (uint64_t c : cores) {
+            Core2 q{c, {}, (int)key};
+            const std::vector<int> &v = I.pairs_by_key[key];
+            for (size_t t = 0; t < v.size(); ++t) {
+                const uint64_t m = (1ULL << I.pair_i[(size_t)v[t]]) | (1ULL << I.pair_j[(size_t)v[t]]);
+                if (c & m) continue;
+                auto it = S.index.find(c | m);
+                if (it != S.index.end()) q.at.push_back({(int)t, it->second});
+            }
+            if (!q.at.empty()) out.push_back(std::move(q));
+        }
+}
+
+template <typename V>
+cudaError_t put_plan(AdjPlan &P, V *&d, const std::vector<V> &h)
+{
+    cudaError_t e = cudaMalloc((void **)&d, std::max<size_t>(1, h.size()) * sizeof(V));
+    if (e != cudaSuccess) return e;
+    P.owned.push_back(d);
+    return h.empty() ? cudaSuccess : cudaMemcpy(d, h.data(), h.size() * sizeof(V), cudaMemcpyHostToDevice);
+}
+
+// Units of the Gram matrices, once per loaded interaction; false (with no error) where they do not apply.
+int build_plan(bs_ctx *c)
+{
+    AdjPlan &P = c->adj;
+    const Basis &B = c->basis;
+    const Interaction &I = c->inter;
+    PairTables own;   // spaces too wide for the pair-core product have no tables of it yet
+    P.tried = true;
+    const int ns = (int)B.st.size();
+    if (B.trunc || ns > 32 || B.dim >= (int64_t)1 << 31) return BS_OK;
+    if (!c->tab.pair.on && B.Z > 0 && B.N > 0) build_pair_tables(B, I, own, -1);
+    const PairTables &R = c->tab.pair.on ? c->tab.pair : own;
+    if (!R.on && B.Z > 0 && B.N > 0) return BS_OK;
+    cudaError_t e;
+    P.ncn = R.ncn;
+    if ((e = put_plan(P, P.colpos, R.colpos)) != cudaSuccess || (e = put_plan(P, P.nsign, R.nsign)) != cudaSuccess) {
+        c->err = std::string("adjoint tables: ") + cudaGetErrorString(e);
+        (void)cudaGetLastError();
+        release_adj(P);
+        return e == cudaErrorMemoryAllocation ? BS_ENOMEM : BS_ECUDA;
+    }
+    struct U { GramUnit u; double cost; };
+    std::vector<U> units;
+    std::vector<GramRow> rows;
+    std::map<std::pair<int64_t, int>, int> tile_of;
+    // one unit per pair of 64-pair tiles; [r0, r0 + n) the records, positions ascending
+    auto add = [&](int64_t out, int np, int r0, int n, int ncol, int64_t stride, int core0) {
+        for (int ja = 0; ja < np; ja += kGramTile)
+            for (int jb = 0; jb < np; jb += kGramTile) {
+                GramUnit u = {};
+                u.out = out + (int64_t)jb * np + ja;
+                u.np = np;
+                u.pa = ja;
+                u.pb = jb;
+                u.ta = std::min(kGramTile, np - ja);
+                u.tb = std::min(kGramTile, np - jb);
+                u.a0 = u.b0 = -1;
+                for (int r = r0; r < r0 + n; ++r) {
+                    const int p = rows[(size_t)r].pos;
+                    if (p >= ja && p < ja + u.ta) { if (u.a0 < 0) u.a0 = r; ++u.na; }
+                    if (p >= jb && p < jb + u.tb) { if (u.b0 < 0) u.b0 = r; ++u.nb; }
+                }
+                if (!u.na || !u.nb) continue;
+                u.ncol = ncol;
+                u.stride = stride;
+                u.core0 = core0;
+                u.tile = tile_of.emplace(std::make_pair(u.out, np), (int)tile_of.size()).first->second;
+                units.push_back(U{u, (double)(ncol + 8) * ((u.ta + 3) / 4) * ((u.tb + 3) / 4) / 256.0 + 2.0});
+            }
+    };
+    int64_t nout = 0;
+    // pn: the matrices of the pair tables
+    P.pn_size = B.Z > 0 && B.N > 0 ? (int64_t)R.w.size() : 0;
+    nout = P.pn_size;
+    if (P.pn_size)
+        for (const PairCore &pc : R.cores)
+            for (int g = 0; g < pc.ngrp; ++g) {
+                const PairGroup &G = R.grps[(size_t)(pc.grp0 + g)];
+                const int r0 = (int)rows.size();
+                for (int r = 0; r < G.nrec; ++r) {
+                    const PairRec &q = R.recs[(size_t)(pc.rec0 + G.rec0 + r)];
+                    rows.push_back(GramRow{(int64_t)q.xoff, (int)(q.wj & 0xFFFFu), (uint8_t)(q.wj >> 16 & 255u), (uint8_t)(q.srec >> 31), 0});
+                }
+                add(G.woff, G.np, r0, G.nrec, G.ncore, 1, G.core0);
+            }
+    // like particles: pair-key matrices shared by both species
+    P.like_off.clear();
+    for (const std::vector<int> &v : I.pairs_by_key) {
+        P.like_off.push_back(nout);
+        nout += (int64_t)v.size() * (int64_t)v.size();
+    }
+    for (int spc = 0; spc < 2; ++spc) {
+        const Species &S = B.sp[spc];
+        std::vector<Core2> cores;
+        core2_lists(B, I, spc, cores);
+        for (const Core2 &q : cores) {
+            const int sec = S.sec_of_sd[(size_t)q.at[0].second];   // all of a core's SDs for one key share it
+            int blk = -1;
+            if (spc == 0) blk = B.block_of_psec[(size_t)sec];
+            else
+                for (size_t b = 0; b < B.blocks.size(); ++b)
+                    if (B.blocks[b].ns == sec) blk = (int)b;
+            if (blk < 0) continue;
+            const Block &K = B.blocks[(size_t)blk];
+            const std::vector<int> &v = I.pairs_by_key[(size_t)q.key];
+            const int r0 = (int)rows.size();
+            for (const auto &e : q.at) {
+                const int k = I.pair_i[(size_t)v[(size_t)e.first]], l = I.pair_j[(size_t)v[(size_t)e.first]];
+                const uint64_t m = S.bits[(size_t)e.second];
+                const bool neg = (sgn_below(m, k) < 0) != (sgn_below(m & ~(1ULL << k), l) < 0);
+                const int64_t loc = e.second - S.sec[(size_t)sec].start;
+                rows.push_back(GramRow{K.off + loc * (spc == 0 ? K.nN : 1), e.first, 0, (uint8_t)neg, 0});
+            }
+            add(P.like_off[(size_t)q.key], (int)v.size(), r0, (int)q.at.size(), (int)(spc == 0 ? K.nN : K.nP), spc == 0 ? 1 : K.nN, -1);
+        }
+    }
+    P.pd = nout;
+    nout += (int64_t)B.sp[0].bits.size();
+    P.nd = nout;
+    nout += (int64_t)B.sp[1].bits.size();
+    P.nout = nout;
+    // by matrix, then shared out to the CTAs (two per SM) in consecutive parts of equal cost
+    std::stable_sort(units.begin(), units.end(), [](const U &a, const U &b) { return a.u.tile < b.u.tile; });
+    int nsm = 152;
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) (void)cudaGetLastError();
+    double total = 0.0;
+    for (const U &u : units) total += u.cost;
+    const int parts = (int)std::min<size_t>((size_t)nsm * 2, units.size());
+    std::vector<int> range(1, 0);
+    std::vector<GramUnit> gu;
+    double run = 0.0;
+    for (const U &u : units) {
+        if (!gu.empty() && (int)range.size() < parts && run + 0.5 * u.cost >= total * (double)range.size() / parts) range.push_back((int)gu.size());
+        run += u.cost;
+        gu.push_back(u.u);
+    }
+    range.push_back((int)gu.size());
+    P.nctas = gu.empty() ? 0 : (int)range.size() - 1;
+    std::vector<int4> nt;
+    for (size_t b = 0; b < B.blocks.size(); ++b)
+        for (int64_t r = 0; r < B.blocks[b].nP; r += kNdRows)
+            for (int64_t q = 0; q < B.blocks[b].nN; q += 128) nt.push_back(make_int4((int)b, (int)r, (int)q, 0));
+    P.nnd = (int)nt.size();
+    // where every pn density belongs in the W_pn layout
+    P.pn_to_w.assign((size_t)P.pn_size, -1);
+    if (P.pn_size) {
+        std::map<std::pair<int, int>, std::vector<std::pair<int, int>>> pairs;
+        for (int i = 0; i < ns; ++i)
+            for (int j = 0; j < ns; ++j)
+                pairs[{B.st[(size_t)i].twom + B.st[(size_t)j].twom, B.st[(size_t)i].par ^ B.st[(size_t)j].par}].push_back({i, j});
+        int64_t w = 0;   // the matrices in the order of the keys, as build_pair_tables lays them out
+        for (const auto &kv : pairs)
+            for (const auto &kl : kv.second)
+                for (const auto &ij : kv.second) {
+                    const int op = ij.first * ns + kl.first, on = ij.second * ns + kl.second;
+                    const int g = I.ops.group_of_op[(size_t)op], h = g < 0 ? -1 : I.conj_group[(size_t)g];
+                    if (h >= 0 && I.ops.group_of_op[(size_t)on] == h)
+                        P.pn_to_w[(size_t)w] = I.wpn_off[(size_t)g] + (int64_t)I.ops.local_of_op[(size_t)op] * (int64_t)I.ops.ops[(size_t)h].size() +
+                                               I.ops.local_of_op[(size_t)on];
+                    ++w;
+                }
+    }
+    if ((e = put_plan(P, P.units, gu)) != cudaSuccess || (e = put_plan(P, P.rows, rows)) != cudaSuccess ||
+        (e = put_plan(P, P.range, range)) != cudaSuccess || (e = put_plan(P, P.ndtasks, nt)) != cudaSuccess ||
+        (e = put_plan(P, P.out, std::vector<double>((size_t)nout, 0.0))) != cudaSuccess ||
+        (e = cudaMallocHost((void **)&P.host, (size_t)nout * sizeof(double))) != cudaSuccess) {
+        c->err = std::string("adjoint tables: ") + cudaGetErrorString(e);
+        (void)cudaGetLastError();
+        release_adj(P);
+        return e == cudaErrorMemoryAllocation ? BS_ENOMEM : BS_ECUDA;
+    }
+    P.on = true;
+    return BS_OK;
+}
+
+// gtheta from the Gram matrices
+int gram_backward(bs_ctx *c, const void *x, const void *gy, double *gtheta, int k, bs_dtype dt, cudaStream_t s)
+{
+    AdjPlan &P = c->adj;
+    const Interaction &I = c->inter;
+    const Basis &B = c->basis;
+    cudaError_t e = cudaMemsetAsync(P.out, 0, (size_t)P.nout * sizeof(double), s);
+    if (e == cudaSuccess) {
+        if (dt == BS_F64) {
+            const double *xi = (const double *)x, *gi = (const double *)gy;
+            e = k == 1 ? launch_gram<double, 1>(c, xi, gi, s) : k == 2 ? launch_gram<double, 2>(c, xi, gi, s)
+              : k == 4 ? launch_gram<double, 4>(c, xi, gi, s) : launch_gram<double, 8>(c, xi, gi, s);
+        } else {
+            const float *xi = (const float *)x, *gi = (const float *)gy;
+            e = k == 1 ? launch_gram<float, 1>(c, xi, gi, s) : k == 2 ? launch_gram<float, 2>(c, xi, gi, s)
+              : k == 4 ? launch_gram<float, 4>(c, xi, gi, s) : launch_gram<float, 8>(c, xi, gi, s);
+        }
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(P.host, P.out, (size_t)P.nout * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        c->err = std::string("adjoint: ") + cudaGetErrorString(e);
+        return BS_ECUDA;
+    }
+    const int ns = (int)B.st.size(), no = (int)c->spe_in.size();
+    std::vector<double> n1((size_t)ns, 0.0);
+    for (int spc = 0; spc < 2; ++spc) {
+        const double *d = P.host + (spc == 0 ? P.pd : P.nd);
+        for (size_t g = 0; g < B.sp[spc].bits.size(); ++g)
+            for (uint64_t m = B.sp[spc].bits[g]; m; m &= m - 1) n1[(size_t)__builtin_ctzll(m)] += d[g];
+    }
+    for (int st = 0; st < ns; ++st) gtheta[B.st[(size_t)st].orb] += n1[(size_t)st];
+    std::vector<double> rho2((size_t)I.npairs * I.npairs, 0.0), rho(I.Wpn.size(), 0.0);
+    for (size_t key = 0; key < I.pairs_by_key.size(); ++key) {
+        const std::vector<int> &v = I.pairs_by_key[key];
+        const double *m = P.host + P.like_off[key];
+        for (size_t b = 0; b < v.size(); ++b)   // row kl, column ij
+            for (size_t a = 0; a < v.size(); ++a) rho2[(size_t)v[a] * I.npairs + (size_t)v[b]] = m[b * v.size() + a];
+    }
+    for (int64_t i = 0; i < P.pn_size; ++i)
+        if (P.pn_to_w[(size_t)i] >= 0) rho[(size_t)P.pn_to_w[(size_t)i]] = P.host[i];
+    for (const WTerm &t : c->dWpp) gtheta[no + t.t] += rho2[(size_t)t.at] * t.c;
+    for (const WTerm &t : c->dWpn) gtheta[no + t.t] += rho[(size_t)t.at] * t.c;
     return BS_OK;
 }
 
 }  // namespace
+
+void release_adj(AdjPlan &P)
+{
+    for (void *p : P.owned) cudaFree(p);
+    if (P.host) cudaFreeHost(P.host);
+    P = AdjPlan();
+}
 
 int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gtheta, int k, bs_dtype dt,
                  void *stream)
@@ -254,7 +699,12 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
     cudaStream_t s = (cudaStream_t)stream;
     int rc = launch_hx(c, gy, gx, k, dt, stream, c->err);   // gx = H gy (H symmetric)
     if (rc || !gtheta) return rc;
-    if (!c->have_dW && (rc = build_derivatives(c))) return rc;
+    if (!c->have_dW) {
+        build_interaction_derivatives(c->basis, c->inter, c->tbme_in, c->dWpp, c->dWpn);
+        c->have_dW = true;
+    }
+    if (!c->adj.tried && (rc = build_plan(c))) return rc;
+    if (c->adj.on) return gram_backward(c, x, gy, gtheta, k, dt, s);
     const Tables &T = c->tab;
     const Interaction &I = c->inter;
     cudaError_t e;
@@ -305,12 +755,8 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
     split_like(c->basis, I, 1, T.nn, gnn, rho2, rho1n);
     const int no = (int)c->spe_in.size();
     for (int st = 0; st < ns; ++st) gtheta[c->basis.st[(size_t)st].orb] += rho1p[st] + rho1n[st];
-    for (size_t t = 0; t < c->tbme_in.size(); ++t) {
-        double g = 0.0;
-        for (const auto &kv : c->dWpp[t]) g += rho2[(size_t)kv.first] * kv.second;
-        for (const auto &kv : c->dWpn[t]) g += rho[(size_t)kv.first] * kv.second;
-        gtheta[no + t] += g;
-    }
+    for (const WTerm &t : c->dWpp) gtheta[no + t.t] += rho2[(size_t)t.at] * t.c;
+    for (const WTerm &t : c->dWpn) gtheta[no + t.t] += rho[(size_t)t.at] * t.c;
     return BS_OK;
 }
 

@@ -370,6 +370,7 @@ void bs_destroy(bs_ctx *c)
     if (c->device >= 0) {
         cudaSetDevice(c->device);
         release(c->dev);
+        release_adj(c->adj);
         if (c->adj_gpp) cudaFree(c->adj_gpp);
         if (c->adj_gnn) cudaFree(c->adj_gnn);
         if (c->adj_rho) cudaFree(c->adj_rho);
@@ -476,7 +477,8 @@ int bs_load_interaction(bs_ctx *c, const double *spe, int n_spe, const bs_tbme *
         rc = build_tables(c->basis, c->inter, c->tab, c->err, nsm);
         if (rc) return rc;
         if (c->device >= 0) {
-                if (c->adj_gpp) { cudaFree(c->adj_gpp); cudaFree(c->adj_gnn); cudaFree(c->adj_rho); }
+            release_adj(c->adj);
+            if (c->adj_gpp) { cudaFree(c->adj_gpp); cudaFree(c->adj_gnn); cudaFree(c->adj_rho); }
             c->adj_gpp = c->adj_gnn = c->adj_rho = nullptr;
             rc = upload(c->basis, c->inter, c->tab, c->dev, c->err);
             if (rc) { release(c->dev); return rc; }

@@ -96,7 +96,90 @@ struct Tbme {
     }
 };
 
+// <ja mi jb mj | J M> of every pair of states (i, j) and J = 0 .. nJ - 1
+std::vector<double> pair_amplitudes(const Basis &B, int nJ)
+{
+    const int ns = (int)B.st.size();
+    auto tj = [&](int s) { return B.orb_twoj[B.st[s].orb]; };
+    std::vector<double> Q((size_t)ns * ns * nJ, 0.0);
+    for (int i = 0; i < ns; ++i)
+        for (int j = 0; j < ns; ++j)
+            for (int J = 0; J < nJ; ++J)
+                Q[((size_t)i * ns + j) * nJ + J] = clebsch(tj(i), B.st[i].twom, tj(j), B.st[j].twom, 2 * J, B.st[i].twom + B.st[j].twom);
+    return Q;
+}
+
 }  // namespace
+
+// The same sums as build_interaction, per matrix element: dW/dV of every element as given, one pass over the
+// M-scheme elements (each names the at most 2 (j_max + 1) coupled ones it contains).
+void build_interaction_derivatives(const Basis &B, const Interaction &I, const std::vector<bs_tbme> &tbme, std::vector<WTerm> &like,
+                                   std::vector<WTerm> &pn)
+{
+    like.clear();
+    pn.clear();
+    const std::vector<SpState> &st = B.st;
+    const int ns = (int)st.size(), no = (int)B.orb_twoj.size();
+    int nJ = 1;
+    for (int a = 0; a < no; ++a) nJ = std::max(nJ, B.orb_twoj[a] + 1);
+    Tbme V;   // for its phases
+    V.B = &B;
+    // element by canonical label: its place in the list and the sign of the value as given
+    std::vector<std::pair<int, double>> of((size_t)2 * nJ * no * no * no * no, {-1, 0.0});
+    auto at = [&](int T, int J, int a, int b, int c, int d) -> std::pair<int, double> & {
+        return of[((((((size_t)T * nJ + J) * no + a) * no + b) * no + c) * no + d)];
+    };
+    for (size_t t = 0; t < tbme.size(); ++t) {
+        int a = tbme[t].a - 1, b = tbme[t].b - 1, c = tbme[t].c - 1, d = tbme[t].d - 1;
+        const int J = tbme[t].J, T = tbme[t].T;
+        double ph = 1.0;
+        if (a > b) { ph *= V.phase(a, b, J, T); std::swap(a, b); }
+        if (c > d) { ph *= V.phase(c, d, J, T); std::swap(c, d); }
+        if (std::make_pair(a, b) > std::make_pair(c, d)) { std::swap(a, c); std::swap(b, d); }
+        at(T, J, a, b, c, d) = {(int)t, ph};
+    }
+    auto find = [&](int T, int J, int a, int b, int c, int d) -> std::pair<int, double> {
+        double ph = 1.0;
+        if (a > b) { ph *= V.phase(a, b, J, T); std::swap(a, b); }
+        if (c > d) { ph *= V.phase(c, d, J, T); std::swap(c, d); }
+        if (std::make_pair(a, b) > std::make_pair(c, d)) { std::swap(a, c); std::swap(b, d); }
+        const std::pair<int, double> &e = at(T, J, a, b, c, d);
+        return {e.first, e.first < 0 ? 0.0 : ph * e.second};
+    };
+    const std::vector<double> Q = pair_amplitudes(B, nJ);
+    auto q = [&](int i, int j, int J) { return Q[((size_t)i * ns + j) * nJ + J]; };
+    for (const std::vector<int> &grp : I.pairs_by_key)
+        for (int p : grp)
+            for (int r : grp) {
+                const int i = I.pair_i[p], j = I.pair_j[p], k = I.pair_i[r], l = I.pair_j[r];
+                const double z = (st[i].orb == st[j].orb ? std::sqrt(2.0) : 1.0) * (st[k].orb == st[l].orb ? std::sqrt(2.0) : 1.0);
+                for (int J = 0; J < nJ; ++J) {
+                    const double v = z * q(i, j, J) * q(k, l, J);
+                    if (v == 0.0) continue;
+                    const auto e = find(1, J, st[i].orb, st[j].orb, st[k].orb, st[l].orb);
+                    if (e.first >= 0) like.push_back(WTerm{(int64_t)p * I.npairs + r, e.first, v * e.second});
+                }
+            }
+    for (size_t g = 0; g < I.ops.ops.size(); ++g) {
+        const int h = I.conj_group[g];
+        if (h < 0) continue;
+        const size_t nb = I.ops.ops[(size_t)h].size();
+        for (size_t ia = 0; ia < I.ops.ops[g].size(); ++ia)
+            for (size_t ib = 0; ib < nb; ++ib) {
+                const int i = I.ops.ops[g][ia] / ns, k = I.ops.ops[g][ia] % ns, j = I.ops.ops[(size_t)h][ib] / ns, l = I.ops.ops[(size_t)h][ib] % ns;
+                const int a = st[i].orb, b = st[j].orb, c = st[k].orb, d = st[l].orb;
+                const double z = 0.5 * (a == b ? std::sqrt(2.0) : 1.0) * (c == d ? std::sqrt(2.0) : 1.0);
+                for (int J = 0; J < nJ; ++J) {
+                    const double v = z * q(i, j, J) * q(k, l, J);
+                    if (v == 0.0) continue;
+                    for (int T = 0; T < 2; ++T) {
+                        const auto e = find(T, J, a, b, c, d);
+                        if (e.first >= 0) pn.push_back(WTerm{I.wpn_off[g] + (int64_t)(ia * nb + ib), e.first, v * e.second});
+                    }
+                }
+            }
+    }
+}
 
 int OpGroups::find(int dtwom, int dpar) const
 {
@@ -208,11 +291,7 @@ int build_interaction(const Basis &B, const double *spe, int n_spe, const bs_tbm
         I.wpn_off[g + 1] = I.wpn_off[g] + (h < 0 ? 0 : (int64_t)G.ops[g].size() * (int64_t)G.ops[h].size());
     }
     // pn amplitudes Q_J(ij) = <ja mi jb mj | J M>, i proton, j neutron
-    std::vector<double> Q((size_t)ns * ns * nJ, 0.0);
-    for (int i = 0; i < ns; ++i)
-        for (int j = 0; j < ns; ++j)
-            for (int J = 0; J < nJ; ++J)
-                Q[((size_t)i * ns + j) * nJ + J] = clebsch(tj(i), st[i].twom, tj(j), st[j].twom, 2 * J, st[i].twom + st[j].twom);
+    const std::vector<double> Q = pair_amplitudes(B, nJ);
     I.Wpn.assign((size_t)I.wpn_off[ng], 0.0);
     for (int g = 0; g < ng; ++g) {
         int h = I.conj_group[g];

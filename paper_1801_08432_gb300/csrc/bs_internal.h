@@ -352,6 +352,44 @@ struct DevLLink {
     int64_t ptr_off;        // class CSR in ppx_ptr / nnx_ptr
 };
 
+// Derivative of the decoupled elements: W[at] += c dV[t] (Wpp: pair * npairs + pair; Wpn).
+struct WTerm {
+    int64_t at;
+    int t;
+    double c;
+};
+
+// Gram matrices of the adjoint (bs_adjoint.cu).
+struct GramRow {            // a pair in a unit: first element, place in the matrix, neutron state (pn), sign
+    int64_t off;
+    int pos;
+    uint8_t l, sign;
+    uint16_t pad;
+};
+struct GramUnit {
+    int64_t out;            // first entry of its matrix tile
+    int64_t stride;         // between columns (pp 1, nn the block's width)
+    int tile, np;           // tile number; width of the matrix
+    int ta, tb, pa, pb;     // rows (kl: tb) and columns (ij: ta) of the tile, and the first position of each
+    int a0, na, b0, nb;     // records of the pairs ij and kl
+    int ncol, core0;        // columns; pn: first neutron core, else -1
+};
+struct AdjPlan {
+    bool tried = false, on = false;
+    GramUnit *units = nullptr;
+    GramRow *rows = nullptr;
+    int *range = nullptr;
+    int4 *ndtasks = nullptr;
+    uint16_t *colpos = nullptr;   // neutron cores, as PairTables
+    uint32_t *nsign = nullptr;
+    int ncn = 0;
+    double *out = nullptr, *host = nullptr;   // pn matrices, like matrices, overlaps per proton and neutron SD
+    int nctas = 0, nnd = 0;
+    int64_t pn_size = 0, pd = 0, nd = 0, nout = 0;
+    std::vector<int64_t> like_off, pn_to_w;
+    std::vector<void *> owned;
+};
+
 struct DevTask {            // one CTA: destination block, proton row, column tile
     int block;
     int row;
@@ -470,8 +508,9 @@ struct bs_ctx {
     std::vector<bs_tbme> tbme_in;
     // adjoint: derivative of the decoupled tables w.r.t. each TBME, sparse, built on first use
     bool have_dW = false;
-    std::vector<std::vector<std::pair<int64_t, double>>> dWpp, dWpn;
-    // adjoint device buffers
+    std::vector<bs::WTerm> dWpp, dWpn;
+    bs::AdjPlan adj;
+    // adjoint device buffers of the spaces without Gram matrices
     double *adj_gpp = nullptr, *adj_gnn = nullptr, *adj_rho = nullptr;
 };
 
@@ -481,6 +520,9 @@ int build_basis(Basis &B, const bs_orbit *orbits, int n_orbits, int Z, int N, in
                 std::string &err);
 int build_interaction(const Basis &B, const double *spe, int n_spe, const bs_tbme *tbme, int n_tbme,
                       Interaction &I, std::string &err);
+void build_interaction_derivatives(const Basis &B, const Interaction &I, const std::vector<bs_tbme> &tbme, std::vector<WTerm> &like,
+                                   std::vector<WTerm> &pn);
+void release_adj(AdjPlan &P);
 int build_tables(const Basis &B, const Interaction &I, Tables &T, std::string &err, int grid = 152);
 void build_like_lists(const Basis &B, int spc, const LikeJumps &L, const LikeCross &X, LikeLists &O);
 void build_like_panels(const Basis &B, int spc, int pos, LikePanels &O);
