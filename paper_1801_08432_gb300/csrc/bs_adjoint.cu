@@ -235,7 +235,9 @@ constexpr int kGramTile = 64;          // at most 64 x 64 pairs: 16 x 16 threads
 struct GramArgs {
     const GramUnit *units;
     const GramRow *rows;
-    const int *range;                  // units of CTA b: range[b] .. range[b + 1] - 1
+    const int *range;                  // batch b: units range[b] .. range[b + 1] - 1
+    int nbatch;
+    int *next;                         // batches claimed beyond the grid's first ones (zero before the launch)
     const uint16_t *colpos;            // neutron cores (bs_pair.cpp)
     const uint32_t *nsign;
     int ncn;
@@ -263,6 +265,30 @@ struct GramSum<float> {
     __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
 };
 
+// K values of a staged element, in 16-byte accesses where it is that wide
+template <typename T, int K>
+__device__ __forceinline__ void gget(const T *p, T (&v)[K])
+{
+    if constexpr (K * sizeof(T) >= 16) {
+#pragma unroll
+        for (int q = 0; q < K; q += 16 / (int)sizeof(T)) *reinterpret_cast<int4 *>(v + q) = *reinterpret_cast<const int4 *>(p + q);
+    } else {
+#pragma unroll
+        for (int q = 0; q < K; ++q) v[q] = p[q];
+    }
+}
+template <typename T, int K>
+__device__ __forceinline__ void gput(T *p, const T (&v)[K])
+{
+    if constexpr (K * sizeof(T) >= 16) {
+#pragma unroll
+        for (int q = 0; q < K; q += 16 / (int)sizeof(T)) *reinterpret_cast<int4 *>(p + q) = *reinterpret_cast<const int4 *>(v + q);
+    } else {
+#pragma unroll
+        for (int q = 0; q < K; ++q) p[q] = v[q];
+    }
+}
+
 // rho(ij,kl) += sum over a unit's columns (pn: neutron cores of one group;
 // pp: neutron SDs; nn: proton SDs) of gy[ij] . x[kl].  A CTA stages the two
 // [pairs][columns][K] tiles in shared memory, each element once and with its
@@ -270,7 +296,7 @@ struct GramSum<float> {
 // pairs per thread, in registers over all of the CTA's consecutive units of
 // one matrix (units are ordered by matrix).  (ceil(np / 4))^2 threads cover a
 // matrix; a small one is covered several times, by slices that take every
-// S-th column.  FP32 add issue bounds it (K multiply-adds and 7 adds per
+// S-th column.  CTAs claim batches of units from a counter.  FP32 add issue bounds it (K multiply-adds and 7 adds per
 // pair and column), against one FP64 shared-memory atomic per pair of jumps
 // before: 48Cr k = 4, 26.7 ms for pn alone.
 template <typename T, int K>
@@ -278,11 +304,14 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
                                                             double *__restrict__ rho)
 {
     constexpr int E = K * (int)sizeof(T);                 // bytes of an element
-    constexpr int CH = 256 / E;                           // columns staged at a time
+    constexpr int LG = E == 4 ? 6 : E == 8 ? 5 : E == 16 ? 4 : E == 32 ? 3 : 2;   // 2^LG columns of 128 pairs fit
     constexpr int PAD = E < 16 ? K : 16 / (int)sizeof(T);   // neighbouring pairs' elements lie in other banks
-    constexpr int LD = CH * K + PAD;
-    __shared__ __align__(16) T sx[kGramTile * LD], sg[kGramTile * LD];
-    __shared__ int rowa[kGramTile], rowb[kGramTile];      // record of a tile's pair, -1: not in this unit
+    __shared__ __align__(16) T tiles[2 * kGramTile * ((1 << LG) * K + PAD)];   // gy's pairs, then x's
+    __shared__ int claim;
+    // per pair of the two tiles (gy's, then x's): first element, and l | sign << 8, -1 where the unit lacks it
+    __shared__ int64_t roff[2 * kGramTile];
+    __shared__ int rl[2 * kGramTile];
+    constexpr int NB = E <= 16 ? 8 : 128 / E;             // elements a thread has on the way at a time
     const int tid = threadIdx.x;
     GramSum<T> acc[4][4];
     int out = -1, ga = 1, gb = 1, np = 0, ta = 0, tb = 0;   // the matrix tile the sums belong to
@@ -301,7 +330,8 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
                 }
         }
     };
-    for (int u = A.range[blockIdx.x]; u < A.range[blockIdx.x + 1]; ++u) {
+    for (int batch = blockIdx.x; batch < A.nbatch;) {
+    for (int u = A.range[batch]; u < A.range[batch + 1]; ++u) {
         const GramUnit U = A.units[u];
         if (U.tile != out) {
             flush();
@@ -317,65 +347,89 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
             ga = (ta + 3) / 4;
             gb = (tb + 3) / 4;
         }
+        // small tiles leave room for more columns at a time
+        int lg = LG;
+        const int na = 4 * ga, nall = na + 4 * gb;   // staged rows: every thread has four of each tile, absent ones zero
+        while (nall << (lg + 1 - LG) <= 2 * kGramTile) ++lg;
+        const int CH = 1 << lg, LD = CH * K + PAD;
+        const T *sg = tiles, *sx = tiles + na * LD;
         const int nt = ga * gb, S = kGramThreads / nt;
         const int slice = tid / nt, t = tid % nt, ia = t % ga, ib = t / ga;
         __syncthreads();   // the last unit's tiles and records are read
-        if (tid < kGramTile) rowa[tid] = rowb[tid] = -1;
+        if (tid < 2 * kGramTile) rl[tid] = -1;
         __syncthreads();
-        for (int r = tid; r < U.na; r += kGramThreads) rowa[A.rows[U.a0 + r].pos - U.pa] = U.a0 + r;
-        for (int r = tid; r < U.nb; r += kGramThreads) rowb[A.rows[U.b0 + r].pos - U.pb] = U.b0 + r;
+        for (int r = tid; r < U.na + U.nb; r += kGramThreads) {
+            const bool isx = r >= U.na;
+            const GramRow R = A.rows[isx ? U.b0 + r - U.na : U.a0 + r];
+            const int slot = isx ? na + R.pos - U.pb : R.pos - U.pa;
+            roff[slot] = R.off;
+            rl[slot] = R.l | R.sign << 8;
+        }
         __syncthreads();
         for (int c0 = 0; c0 < U.ncol; c0 += CH) {
             if (c0) __syncthreads();
-            for (int n = tid; n < (ta + tb) * CH; n += kGramThreads) {
-                const int slot = n / CH, c = n % CH, col = c0 + c;
-                const bool isx = slot >= ta;
-                const int sl = isx ? slot - ta : slot;
-                const int r = isx ? rowb[sl] : rowa[sl];
-                T *d = (isx ? sx : sg) + sl * LD + c * K;
-                int64_t at = -1;
-                bool neg = false;
-                if (r >= 0 && col < U.ncol) {
-                    const GramRow R = A.rows[r];
-                    neg = R.sign;
-                    if (U.core0 >= 0) {   // pn: the column of core + l, and the sign of a+_l on the core
-                        const int p = __ldg(A.colpos + (size_t)R.l * A.ncn + U.core0 + col);
-                        if (p != 0xFFFF) at = R.off + p;
-                        neg = neg != (bool)(__ldg(A.nsign + U.core0 + col) >> R.l & 1u);
-                    } else {
-                        at = R.off + (int64_t)col * U.stride;
+            // columns first, then elements: NB dependent pairs of loads in flight
+            const int total = nall * CH;
+            for (int n0 = tid; n0 < total; n0 += NB * kGramThreads) {
+                int64_t at[NB];
+                bool neg[NB];
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    const int n = n0 + j * kGramThreads, slot = n >> lg, col = c0 + (n & (CH - 1));
+                    at[j] = -1;
+                    neg[j] = false;
+                    if (n < total && col < U.ncol) {
+                        const int r = rl[slot];
+                        if (r >= 0) {
+                            at[j] = roff[slot];
+                            neg[j] = r >> 8;
+                            if (U.core0 >= 0) {   // pn: the column of core + l, and the sign of a+_l on the core
+                                const int l = r & 255;
+                                const int p = __ldg(A.colpos + (size_t)l * A.ncn + U.core0 + col);
+                                neg[j] = neg[j] != (bool)(__ldg(A.nsign + U.core0 + col) >> l & 1u);
+                                at[j] = p == 0xFFFF ? -1 : at[j] + p;
+                            } else {
+                                at[j] += (int64_t)col * U.stride;
+                            }
+                        }
                     }
                 }
-                T v[K];
+                alignas(16) T v[NB][K];
 #pragma unroll
-                for (int q = 0; q < K; ++q) v[q] = T(0);
-                if (at >= 0) {
-                    const T *s = (isx ? x : gy) + at * K;
-                    if constexpr (E >= 16) {
+                for (int j = 0; j < NB; ++j) {
+                    const int slot = (n0 + j * kGramThreads) >> lg;
 #pragma unroll
-                        for (int q = 0; q < K; q += 16 / (int)sizeof(T))
-                            *reinterpret_cast<int4 *>(v + q) = __ldg(reinterpret_cast<const int4 *>(s + q));
-                    } else {
+                    for (int q = 0; q < K; ++q) v[j][q] = T(0);
+                    if (at[j] >= 0) {
+                        const T *s = (slot >= na ? x : gy) + at[j] * K;
+                        if constexpr (E >= 16) {
 #pragma unroll
-                        for (int q = 0; q < K; ++q) v[q] = __ldg(s + q);
+                            for (int q = 0; q < K; q += 16 / (int)sizeof(T))
+                                *reinterpret_cast<int4 *>(v[j] + q) = __ldg(reinterpret_cast<const int4 *>(s + q));
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < K; ++q) v[j][q] = __ldg(s + q);
+                        }
                     }
                 }
 #pragma unroll
-                for (int q = 0; q < K; ++q) d[q] = neg ? -v[q] : v[q];
+                for (int j = 0; j < NB; ++j) {
+                    const int n = n0 + j * kGramThreads, slot = n >> lg, c = n & (CH - 1);
+                    if (n >= total) continue;
+#pragma unroll
+                    for (int q = 0; q < K; ++q) v[j][q] = neg[j] ? -v[j][q] : v[j][q];
+                    gput<T, K>(tiles + slot * LD + c * K, v[j]);
+                }
             }
             __syncthreads();
             const int cn = min(CH, U.ncol - c0);
             if (slice < S) {
                 for (int c = slice; c < cn; c += S) {
-                    T a[4][K], b[4][K];
+                    alignas(16) T a[4][K], b[4][K];
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
-                        const T *pa = sg + (ia + ga * p) * LD + c * K, *pb = sx + (ib + gb * p) * LD + c * K;
-#pragma unroll
-                        for (int q = 0; q < K; ++q) {
-                            a[p][q] = pa[q];
-                            b[p][q] = pb[q];
-                        }
+                        gget<T, K>(sg + (ia + ga * p) * LD + c * K, a[p]);
+                        gget<T, K>(sx + (ib + gb * p) * LD + c * K, b[p]);
                     }
 #pragma unroll
                     for (int p = 0; p < 4; ++p)
@@ -389,6 +443,12 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
                 }
             }
         }
+    }
+        // the next batch: a counter shared by the CTAs
+        __syncthreads();
+        if (tid == 0) claim = (int)gridDim.x + atomicAdd(A.next, 1);
+        __syncthreads();
+        batch = claim;
     }
     flush();
 }
@@ -433,8 +493,8 @@ cudaError_t launch_gram(bs_ctx *c, const T *x, const T *gy, cudaStream_t s)
 {
     const AdjPlan &P = c->adj;
     const Device &D = c->dev;
-    GramArgs A{P.units, P.rows, P.range, P.colpos, P.nsign, P.ncn};
-    if (P.nctas > 0) adj_gram<T, K><<<P.nctas, kGramThreads, 0, s>>>(A, x, gy, P.out);
+    GramArgs A{P.units, P.rows, P.range, P.nbatch, reinterpret_cast<int *>(P.out + P.nout), P.colpos, P.nsign, P.ncn};
+    if (P.nbatch > 0) adj_gram<T, K><<<std::min(P.nbatch, P.nctas), kGramThreads, 0, s>>>(A, x, gy, P.out);
     adj_pdiag<T, K><<<(D.nrtasks + 3) / 4, 128, 0, s>>>(D.rtasks, D.nrtasks, D.blocks, x, gy, P.out + P.pd);
     if (P.nnd > 0) adj_ndiag<T, K><<<P.nnd, 128, 0, s>>>(P.ndtasks, D.blocks, x, gy, P.out + P.nd);
     return cudaGetLastError();
@@ -530,7 +590,9 @@ int build_plan(bs_ctx *c)
                 u.stride = stride;
                 u.core0 = core0;
                 u.tile = tile_of.emplace(std::make_pair(u.out, np), (int)tile_of.size()).first->second;
-                units.push_back(U{u, (double)(ncol + 8) * ((u.ta + 3) / 4) * ((u.tb + 3) / 4) / 256.0 + 2.0});
+                // in cycles: per 2048 staged elements their loads, per column of a thread 16 sums
+                const int cols = 2048 / ((u.ta + 3) / 4 * 4 + (u.tb + 3) / 4 * 4), slices = 256 / (((u.ta + 3) / 4) * ((u.tb + 3) / 4));
+                units.push_back(U{u, 1500.0 * (1 + (ncol + cols - 1) / cols) + 376.0 * ((ncol + slices - 1) / slices)});
             }
     };
     int64_t nout = 0;
@@ -584,13 +646,14 @@ int build_plan(bs_ctx *c)
     P.nd = nout;
     nout += (int64_t)B.sp[1].bits.size();
     P.nout = nout;
-    // by matrix, then shared out to the CTAs (two per SM) in consecutive parts of equal cost
+    // by matrix, then in batches of about equal cost, eight for each CTA (two per SM)
     std::stable_sort(units.begin(), units.end(), [](const U &a, const U &b) { return a.u.tile < b.u.tile; });
     int nsm = 152;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) (void)cudaGetLastError();
     double total = 0.0;
     for (const U &u : units) total += u.cost;
-    const int parts = (int)std::min<size_t>((size_t)nsm * 2, units.size());
+    P.nctas = nsm * 2;
+    const int parts = (int)std::min<size_t>((size_t)P.nctas * 8, units.size());
     std::vector<int> range(1, 0);
     std::vector<GramUnit> gu;
     double run = 0.0;
@@ -600,7 +663,7 @@ int build_plan(bs_ctx *c)
         gu.push_back(u.u);
     }
     range.push_back((int)gu.size());
-    P.nctas = gu.empty() ? 0 : (int)range.size() - 1;
+    P.nbatch = gu.empty() ? 0 : (int)range.size() - 1;
     std::vector<int4> nt;
     for (size_t b = 0; b < B.blocks.size(); ++b)
         for (int64_t r = 0; r < B.blocks[b].nP; r += kNdRows)
@@ -627,7 +690,7 @@ int build_plan(bs_ctx *c)
     }
     if ((e = put_plan(P, P.units, gu)) != cudaSuccess || (e = put_plan(P, P.rows, rows)) != cudaSuccess ||
         (e = put_plan(P, P.range, range)) != cudaSuccess || (e = put_plan(P, P.ndtasks, nt)) != cudaSuccess ||
-        (e = put_plan(P, P.out, std::vector<double>((size_t)nout, 0.0))) != cudaSuccess ||
+        (e = put_plan(P, P.out, std::vector<double>((size_t)nout + 1, 0.0))) != cudaSuccess ||
         (e = cudaMallocHost((void **)&P.host, (size_t)nout * sizeof(double))) != cudaSuccess) {
         c->err = std::string("adjoint tables: ") + cudaGetErrorString(e);
         (void)cudaGetLastError();
@@ -644,7 +707,7 @@ int gram_backward(bs_ctx *c, const void *x, const void *gy, double *gtheta, int 
     AdjPlan &P = c->adj;
     const Interaction &I = c->inter;
     const Basis &B = c->basis;
-    cudaError_t e = cudaMemsetAsync(P.out, 0, (size_t)P.nout * sizeof(double), s);
+    cudaError_t e = cudaMemsetAsync(P.out, 0, (size_t)(P.nout + 1) * sizeof(double), s);
     if (e == cudaSuccess) {
         if (dt == BS_F64) {
             const double *xi = (const double *)x, *gi = (const double *)gy;

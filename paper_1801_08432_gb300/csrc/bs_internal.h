@@ -383,8 +383,8 @@ struct AdjPlan {
     uint16_t *colpos = nullptr;   // neutron cores, as PairTables
     uint32_t *nsign = nullptr;
     int ncn = 0;
-    double *out = nullptr, *host = nullptr;   // pn matrices, like matrices, overlaps per proton and neutron SD
-    int nctas = 0, nnd = 0;
+    double *out = nullptr, *host = nullptr;   // pn matrices, like matrices, overlaps per proton and neutron SD (out: then the batch counter)
+    int nctas = 0, nbatch = 0, nnd = 0;
     int64_t pn_size = 0, pd = 0, nd = 0, nout = 0;
     std::vector<int64_t> like_off, pn_to_w;
     std::vector<void *> owned;
