@@ -23,6 +23,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <type_traits>
 
 #include "bs_internal.h"
 
@@ -243,26 +244,50 @@ struct GramArgs {
     int ncn;
 };
 
-// One partial sum: FP64, or double-float for FP32 vectors (the FP32 pipe adds
-// a term to hi + lo in 7 operations; one FP64 add takes as long as 60).
+// Two partial sums: FP64, or double-float for FP32 vectors (the FP32 pipe adds
+// two terms to hi + lo in 7 packed operations; one FP64 add takes as long as 60).
 template <typename T>
 struct GramSum;
 template <>
 struct GramSum<double> {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double f) { v += f; }
-    __device__ __forceinline__ double get() const { return v; }
+    double v[2] = {0.0, 0.0};
+    __device__ __forceinline__ void add(double f0, double f1)
+    {
+        v[0] += f0;
+        v[1] += f1;
+    }
+    // K = 1: one fused multiply-add each
+    __device__ __forceinline__ void add_prod(double a0, double a1, double b)
+    {
+        v[0] = fma(a0, b, v[0]);
+        v[1] = fma(a1, b, v[1]);
+    }
+    using Part = double;
+    __device__ __forceinline__ double part(int i) const { return v[i]; }
+    static __device__ __forceinline__ double join(double a, double b) { return a + b; }
+    static __device__ __forceinline__ double value(double a) { return a; }
 };
 template <>
 struct GramSum<float> {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float f)
+    float2 hi = {0.0f, 0.0f}, lo = {0.0f, 0.0f};
+    __device__ __forceinline__ void add(float f0, float f1)
     {
-        const float t = hi + f, b = t - hi;
-        lo += (hi - (t - b)) + (f - b);
+        // two-sums; x - y as fma(y, -1, x), the same rounding
+        const float2 m = make_float2(-1.0f, -1.0f), f = make_float2(f0, f1);
+        const float2 t = __fadd2_rn(hi, f), b = __ffma2_rn(hi, m, t);
+        const float2 e = __ffma2_rn(__ffma2_rn(b, m, t), m, hi), g = __ffma2_rn(b, m, f);
+        lo = __fadd2_rn(lo, __fadd2_rn(e, g));
         hi = t;
     }
-    __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ void add_prod(float a0, float a1, float b) { add(a0 * b, a1 * b); }
+    using Part = float2;   // hi, lo
+    __device__ __forceinline__ float2 part(int i) const { return i ? make_float2(hi.y, lo.y) : make_float2(hi.x, lo.x); }
+    static __device__ __forceinline__ float2 join(float2 a, float2 b)
+    {
+        const float t = a.x + b.x, z = t - a.x;
+        return make_float2(t, a.y + b.y + ((a.x - (t - z)) + (b.x - z)));
+    }
+    static __device__ __forceinline__ double value(float2 a) { return (double)a.x + (double)a.y; }
 };
 
 // K values of a staged element, in 16-byte accesses where it is that wide
@@ -290,82 +315,75 @@ __device__ __forceinline__ void gput(T *p, const T (&v)[K])
 }
 
 // rho(ij,kl) += sum over a unit's columns (pn: neutron cores of one group;
-// pp: neutron SDs; nn: proton SDs) of gy[ij] . x[kl].  A CTA stages the two
+// pp: neutron SDs; nn: proton SDs) of gy[ij] . x[kl], for the pairs ij, kl
+// that the unit's core leaves free.  A CTA stages the two
 // [pairs][columns][K] tiles in shared memory, each element once and with its
-// sign, and every element meets all the pairs of the other tile: 4 x 4
-// pairs per thread, in registers over all of the CTA's consecutive units of
-// one matrix (units are ordered by matrix).  (ceil(np / 4))^2 threads cover a
-// matrix; a small one is covered several times, by slices that take every
-// S-th column.  CTAs claim batches of units from a counter.  FP32 add issue bounds it (K multiply-adds and 7 adds per
-// pair and column), against one FP64 shared-memory atomic per pair of jumps
-// before: 48Cr k = 4, 26.7 ms for pn alone.
+// sign, and every element meets all the pairs of the other tile: a thread
+// keeps 4 x 4 or 4 x 3 pairs in registers, whichever leaves fewer threads
+// without work, and slices of the CTA take every S-th column where one set of
+// threads covers the pairs several times.  A unit's sums are added to the
+// matrix tile in shared memory (FP64), which goes to memory when the CTA's
+// units (ordered by tile, claimed in batches from a counter) leave it.  FP32
+// operations bound it (K multiply-adds and 7 adds per pair and column) or
+// FP64 ones.  48Cr k = 4: 26.7 ms for pn alone with an FP64 shared-memory
+// atomic per pair of jumps, 2.3 ms with every pair of the key in fixed
+// threads, 2.0 ms this way (a third of the FP32 pipe; many small units).
+template <typename T>
+__host__ __device__ constexpr int gram_lg(int e) { return e == 4 ? 6 : e == 8 ? 5 : e == 16 ? 4 : e == 32 ? 3 : 2; }   // 2^lg columns of 128 pairs fit
+template <typename T, int K>
+__host__ __device__ constexpr int gram_pad() { return K * (int)sizeof(T) < 16 ? K : 16 / (int)sizeof(T); }   // neighbouring pairs' elements in other banks
+template <typename T, int K>
+__host__ __device__ constexpr int gram_tile_elems() { return 2 * kGramTile * ((1 << gram_lg<T>(K * (int)sizeof(T))) * K + gram_pad<T, K>()); }
+template <typename T, int K>
+constexpr size_t gram_smem() { return (size_t)kGramTile * kGramTile * 8 + (size_t)gram_tile_elems<T, K>() * sizeof(T); }
+
 template <typename T, int K>
 __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T *__restrict__ x, const T *__restrict__ gy,
                                                             double *__restrict__ rho)
 {
     constexpr int E = K * (int)sizeof(T);                 // bytes of an element
-    constexpr int LG = E == 4 ? 6 : E == 8 ? 5 : E == 16 ? 4 : E == 32 ? 3 : 2;   // 2^LG columns of 128 pairs fit
-    constexpr int PAD = E < 16 ? K : 16 / (int)sizeof(T);   // neighbouring pairs' elements lie in other banks
-    __shared__ __align__(16) T tiles[2 * kGramTile * ((1 << LG) * K + PAD)];   // gy's pairs, then x's
+    constexpr int LG = gram_lg<T>(E), PAD = gram_pad<T, K>();
+    extern __shared__ __align__(16) unsigned char gsm[];
+    double *mat = reinterpret_cast<double *>(gsm);        // the tile's sums, [kl][ij]
+    T *tiles = reinterpret_cast<T *>(mat + kGramTile * kGramTile);   // gy's pairs, then x's
     __shared__ int claim;
-    // per pair of the two tiles (gy's, then x's): first element, and l | sign << 8, -1 where the unit lacks it
+    // per pair of the two tiles (gy's, then x's): first element, l | sign << 8 (-1: none), place in the matrix tile
     __shared__ int64_t roff[2 * kGramTile];
-    __shared__ int rl[2 * kGramTile];
+    __shared__ int rl[2 * kGramTile], rp[2 * kGramTile];
     constexpr int NB = E <= 16 ? 8 : 128 / E;             // elements a thread has on the way at a time
     const int tid = threadIdx.x;
-    GramSum<T> acc[4][4];
-    int out = -1, ga = 1, gb = 1, np = 0, ta = 0, tb = 0;   // the matrix tile the sums belong to
+    int out = -1, np = 0, ta = 0, tb = 0;                 // the matrix tile the sums belong to
     int64_t out_at = 0;
-    auto flush = [&]() {
-        if (out < 0) return;
-        const int t = tid % (ga * gb), ia = t % ga, ib = t / ga;
-        if (tid < kGramThreads / (ga * gb) * (ga * gb)) {
-#pragma unroll
-            for (int p = 0; p < 4; ++p)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int a = ia + ga * p, b = ib + gb * q;
-                    const double v = acc[p][q].get();
-                    if (a < ta && b < tb && v != 0.0) atomicAdd(rho + out_at + (int64_t)b * np + a, v);
-                }
+    auto leave = [&]() {   // (every thread, between barriers)
+        for (int i = tid; i < kGramTile * kGramTile; i += kGramThreads) {
+            const int a = i % kGramTile, b = i / kGramTile;
+            const double v = mat[i];
+            if (out >= 0 && a < ta && b < tb && v != 0.0) atomicAdd(rho + out_at + (int64_t)b * np + a, v);
+            mat[i] = 0.0;
         }
     };
-    for (int batch = blockIdx.x; batch < A.nbatch;) {
-    for (int u = A.range[batch]; u < A.range[batch + 1]; ++u) {
-        const GramUnit U = A.units[u];
-        if (U.tile != out) {
-            flush();
-#pragma unroll
-            for (int p = 0; p < 4; ++p)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] = GramSum<T>();
-            out = U.tile;
-            out_at = U.out;
-            np = U.np;
-            ta = U.ta;
-            tb = U.tb;
-            ga = (ta + 3) / 4;
-            gb = (tb + 3) / 4;
-        }
-        // small tiles leave room for more columns at a time
-        int lg = LG;
-        const int na = 4 * ga, nall = na + 4 * gb;   // staged rows: every thread has four of each tile, absent ones zero
+    auto unit = [&](const GramUnit &U, auto rbc) {
+        constexpr int RB = decltype(rbc)::value;
+        const int ga = (U.na + 3) / 4, gb = (U.nb + RB - 1) / RB;
+        const int na = 4 * ga, nall = na + RB * gb;   // staged rows: every thread has 4 and RB, absent ones zero
+        int lg = LG;   // few pairs leave room for more columns at a time
         while (nall << (lg + 1 - LG) <= 2 * kGramTile) ++lg;
         const int CH = 1 << lg, LD = CH * K + PAD;
         const T *sg = tiles, *sx = tiles + na * LD;
         const int nt = ga * gb, S = kGramThreads / nt;
         const int slice = tid / nt, t = tid % nt, ia = t % ga, ib = t / ga;
-        __syncthreads();   // the last unit's tiles and records are read
         if (tid < 2 * kGramTile) rl[tid] = -1;
         __syncthreads();
         for (int r = tid; r < U.na + U.nb; r += kGramThreads) {
             const bool isx = r >= U.na;
             const GramRow R = A.rows[isx ? U.b0 + r - U.na : U.a0 + r];
-            const int slot = isx ? na + R.pos - U.pb : R.pos - U.pa;
+            const int slot = isx ? na + r - U.na : r;
             roff[slot] = R.off;
             rl[slot] = R.l | R.sign << 8;
+            rp[slot] = isx ? R.pos - U.pb : R.pos - U.pa;
         }
         __syncthreads();
+        GramSum<T> acc[2][RB];
         for (int c0 = 0; c0 < U.ncol; c0 += CH) {
             if (c0) __syncthreads();
             // columns first, then elements: NB dependent pairs of loads in flight
@@ -425,32 +443,89 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
             const int cn = min(CH, U.ncol - c0);
             if (slice < S) {
                 for (int c = slice; c < cn; c += S) {
-                    alignas(16) T a[4][K], b[4][K];
+                    alignas(16) T a[4][K], b[RB][K];
 #pragma unroll
-                    for (int p = 0; p < 4; ++p) {
-                        gget<T, K>(sg + (ia + ga * p) * LD + c * K, a[p]);
-                        gget<T, K>(sx + (ib + gb * p) * LD + c * K, b[p]);
-                    }
+                    for (int p = 0; p < 4; ++p) gget<T, K>(sg + (ia + ga * p) * LD + c * K, a[p]);
 #pragma unroll
-                    for (int p = 0; p < 4; ++p)
+                    for (int q = 0; q < RB; ++q) gget<T, K>(sx + (ib + gb * q) * LD + c * K, b[q]);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            T f = a[p][0] * b[q][0];
+                    for (int p = 0; p < 2; ++p)
 #pragma unroll
-                            for (int k = 1; k < K; ++k) f = fma(a[p][k], b[q][k], f);
-                            acc[p][q].add(f);
+                        for (int q = 0; q < RB; ++q) {
+                            if constexpr (K == 1) {
+                                acc[p][q].add_prod(a[2 * p][0], a[2 * p + 1][0], b[q][0]);
+                            } else {
+                                T f0 = a[2 * p][0] * b[q][0], f1 = a[2 * p + 1][0] * b[q][0];
+#pragma unroll
+                                for (int k = 1; k < K; ++k) {
+                                    f0 = fma(a[2 * p][k], b[q][k], f0);
+                                    f1 = fma(a[2 * p + 1][k], b[q][k], f1);
+                                }
+                                acc[p][q].add(f0, f1);
+                            }
                         }
                 }
             }
         }
-    }
+        // slices meet in the tiles' place, [pair of the thread][slice][thread], and are added in order
+        using Part = typename GramSum<T>::Part;
+        Part *part = reinterpret_cast<Part *>(tiles);
+        static_assert(sizeof(Part) * 16 * kGramThreads <= sizeof(T) * gram_tile_elems<T, K>(), "slices' sums do not fit");
+        if (S > 1) {
+            __syncthreads();
+            if (slice < S) {
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int q = 0; q < RB; ++q) part[(p * RB + q) * kGramThreads + tid] = acc[p / 2][q].part(p & 1);
+            }
+            __syncthreads();
+            for (int n = tid; n < 4 * RB * nt; n += kGramThreads) {
+                const int pq = n / nt, th = n % nt;
+                const int a = th % ga + ga * (pq / RB), b = th / ga + gb * (pq % RB);
+                if (a >= U.na || b >= U.nb) continue;
+                Part v = part[pq * kGramThreads + th];
+                for (int sl = 1; sl < S; ++sl) v = GramSum<T>::join(v, part[pq * kGramThreads + sl * nt + th]);
+                mat[rp[na + b] * kGramTile + rp[a]] += GramSum<T>::value(v);
+            }
+        } else if (slice < S) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < RB; ++q) {
+                    const int a = ia + ga * p, b = ib + gb * q;
+                    if (a < U.na && b < U.nb) mat[rp[na + b] * kGramTile + rp[a]] += GramSum<T>::value(acc[p / 2][q].part(p & 1));
+                }
+        }
+        __syncthreads();   // tiles, records and sums are free for the next unit
+    };
+    leave();   // zeros
+    __syncthreads();
+    for (int batch = blockIdx.x; batch < A.nbatch;) {
+        for (int u = A.range[batch]; u < A.range[batch + 1]; ++u) {
+            const GramUnit U = A.units[u];
+            if (U.tile != out) {
+                leave();
+                out = U.tile;
+                out_at = U.out;
+                np = U.np;
+                ta = U.ta;
+                tb = U.tb;
+                __syncthreads();
+            }
+            // 4 x 4 or 4 x 3 pairs a thread: the less work per thread and column
+            const int ga = (U.na + 3) / 4, t4 = ga * ((U.nb + 3) / 4), t3 = ga * ((U.nb + 2) / 3);
+            const int s4 = kGramThreads / t4, s3 = t3 <= kGramThreads ? kGramThreads / t3 : 0;
+            if (s3 > 0 && 3 * s4 <= 4 * s3 && 3 * ((U.ncol + s3 - 1) / s3) < 4 * ((U.ncol + s4 - 1) / s4)) unit(U, std::integral_constant<int, 3>{});
+            else unit(U, std::integral_constant<int, 4>{});
+        }
         // the next batch: a counter shared by the CTAs
-        __syncthreads();
         if (tid == 0) claim = (int)gridDim.x + atomicAdd(A.next, 1);
         __syncthreads();
         batch = claim;
+        __syncthreads();
     }
-    flush();
+    leave();
 }
 
 // Overlaps per SD: pd[g] = gy . x over the other species' SDs of proton SD g, one warp each.
@@ -494,7 +569,12 @@ cudaError_t launch_gram(bs_ctx *c, const T *x, const T *gy, cudaStream_t s)
     const AdjPlan &P = c->adj;
     const Device &D = c->dev;
     GramArgs A{P.units, P.rows, P.range, P.nbatch, reinterpret_cast<int *>(P.out + P.nout), P.colpos, P.nsign, P.ncn};
-    if (P.nbatch > 0) adj_gram<T, K><<<std::min(P.nbatch, P.nctas), kGramThreads, 0, s>>>(A, x, gy, P.out);
+    if (P.nbatch > 0) {
+        constexpr size_t smem = gram_smem<T, K>();
+        const cudaError_t e = cudaFuncSetAttribute(adj_gram<T, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        adj_gram<T, K><<<std::min(P.nbatch, P.nctas), kGramThreads, smem, s>>>(A, x, gy, P.out);
+    }
     adj_pdiag<T, K><<<(D.nrtasks + 3) / 4, 128, 0, s>>>(D.rtasks, D.nrtasks, D.blocks, x, gy, P.out + P.pd);
     if (P.nnd > 0) adj_ndiag<T, K><<<P.nnd, 128, 0, s>>>(P.ndtasks, D.blocks, x, gy, P.out + P.nd);
     return cudaGetLastError();
@@ -590,8 +670,8 @@ int build_plan(bs_ctx *c)
                 u.stride = stride;
                 u.core0 = core0;
                 u.tile = tile_of.emplace(std::make_pair(u.out, np), (int)tile_of.size()).first->second;
-                // in cycles: per 2048 staged elements their loads, per column of a thread 16 sums
-                const int cols = 2048 / ((u.ta + 3) / 4 * 4 + (u.tb + 3) / 4 * 4), slices = 256 / (((u.ta + 3) / 4) * ((u.tb + 3) / 4));
+                // in cycles: a unit's and 2048 staged elements' latency, per column of a thread 16 sums
+                const int cols = 2048 / ((u.na + 3) / 4 * 4 + (u.nb + 3) / 4 * 4), slices = 256 / (((u.na + 3) / 4) * ((u.nb + 3) / 4));
                 units.push_back(U{u, 1500.0 * (1 + (ncol + cols - 1) / cols) + 376.0 * ((ncol + slices - 1) / slices)});
             }
     };
