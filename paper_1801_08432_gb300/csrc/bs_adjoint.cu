@@ -279,7 +279,7 @@ struct GramSum<float> {
         lo = __fadd2_rn(lo, __fadd2_rn(e, g));
         hi = t;
     }
-    __device__ __forceinline__ void add_prod(float a0, float a1, float b) { add(a0 * b, a1 * b); }
+    __device__ __forceinline__ void add_prod(float a0, float a1, float b) { add(__fmul_rn(a0, b), __fmul_rn(a1, b)); }
     using Part = float2;   // hi, lo
     __device__ __forceinline__ float2 part(int i) const { return i ? make_float2(hi.y, lo.y) : make_float2(hi.x, lo.x); }
     static __device__ __forceinline__ float2 join(float2 a, float2 b)

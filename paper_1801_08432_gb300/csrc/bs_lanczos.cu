@@ -199,34 +199,38 @@ __global__ void __launch_bounds__(kDotThreads) blk_dots(const T *__restrict__ V,
     }
 }
 
-// out[e] = sum over CTAs of partial[cta][e], e < n, in a fixed order: thread
-// (slice q, e) adds the CTAs q, q + kRedSl, ... in turn, then the kRedSl
-// slices are added in order.
+// out[e] = sum over CTAs of partial[cta][e], in a fixed order; the partials are doubles or double-floats (float2 hi, lo).
 __device__ __forceinline__ double part_value(double p) { return p; }
 __device__ __forceinline__ double part_value(float2 p) { return (double)p.x + (double)p.y; }
-constexpr int kRedE = 32;   // outputs per CTA
-constexpr int kRedSl = 8;   // slices of the partials per output
+constexpr int kRedE = 4;     // outputs per CTA, one warp each
 
+// Lane q adds the CTAs q, q + 32, ... in order, a fixed shuffle tree the lanes.  FP64 adds bound it (two a cycle and SM, and
+// as slow a conversion), so few outputs share an SM: with 32 outputs to a CTA a 4 x 4 block's 304 partials took 13 us.
 template <typename P>
-__global__ void __launch_bounds__(kRedE * kRedSl) dots_reduce(const P *__restrict__ partial, int ncta, int n,
-                                                              double *__restrict__ out, const int *__restrict__ nb_iter,
-                                                              const int *__restrict__ out_iter, int kk)
+__global__ void __launch_bounds__(kRedE * 32) dots_reduce(const P *__restrict__ partial, int ncta, int n,
+                                                          double *__restrict__ out, const int *__restrict__ nb_iter,
+                                                          const int *__restrict__ out_iter, int kk)
 {
     if (nb_iter) n = (*nb_iter + 1) * kk;       // graph replay: n+1 blocks of k x k
     if (out_iter) out += (int64_t)(*out_iter) * kk;   // graph replay: block n of a history array
-    __shared__ double sl[kRedSl][kRedE];
-    const int el = threadIdx.x % kRedE, q = threadIdx.x / kRedE;
-    const int e = blockIdx.x * kRedE + el;
+    const int lane = threadIdx.x & 31;
+    const int e = blockIdx.x * kRedE + (int)(threadIdx.x >> 5);
+    if (e >= n) return;
     double t = 0.0;
-    if (e < n)
-        for (int c = q; c < ncta; c += kRedSl) t += part_value(partial[(int64_t)c * n + e]);
-    sl[q][el] = t;
-    __syncthreads();
-    if (q == 0 && e < n) {
-        double u = sl[0][el];
-        for (int r = 1; r < kRedSl; ++r) u += sl[r][el];
-        out[e] = u;
+    constexpr int U = 10;   // a lane's loads in flight: all of them for 304 CTAs
+    for (int c0 = lane; c0 < ncta; c0 += U * 32) {
+        P v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int c = c0 + u * 32;
+            v[u] = c < ncta ? partial[(int64_t)c * n + e] : P{};
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) t += part_value(v[u]);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) out[e] = t;
 }
 
 // n_launch: the largest n the launch may see (graph replay reads n from nb_iter)
@@ -234,7 +238,7 @@ template <typename P>
 void reduce_parts(const P *partial, int ncta, int n_launch, int n, double *out, const int *nb_iter, const int *out_iter,
                   int kk, cudaStream_t s)
 {
-    dots_reduce<P><<<(n_launch + kRedE - 1) / kRedE, kRedE * kRedSl, 0, s>>>(partial, ncta, n, out, nb_iter, out_iter, kk);
+    dots_reduce<P><<<(n_launch + kRedE - 1) / kRedE, kRedE * 32, 0, s>>>(partial, ncta, n, out, nb_iter, out_iter, kk);
 }
 
 // W[alpha][j] -= sum_b sum_i V_b[alpha][i] C[b][i][j]   (C: nb blocks of K x K, FP64)
@@ -839,35 +843,16 @@ __global__ void __launch_bounds__(kRsCons + 64, sizeof(T) == 4 ? 2 : 1)
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) sum[0] = R::add(sum[0], R::shfl(sum[0], o));
             } else {
-                if constexpr (std::is_same<T, float>::value) {
-                    DF acc[K];
 #pragma unroll
-                    for (int j = 0; j < K; ++j) acc[j] = DF{0.f, 0.f};
-                    if (!bad) {
+                for (int j = 0; j < K; ++j) sum[j] = 0.0;
+                if (!bad) {
 #pragma unroll
-                        for (int m = 0; m < kRsRT; ++m) {
-                            const int a = r + NR * m;
-                            if (a < rows) {
-                                const float v = tile[a * K + i];
+                    for (int m = 0; m < kRsRT; ++m) {
+                        const int a = r + NR * m;
+                        if (a < rows) {
+                            const double v = (double)tile[a * K + i];
 #pragma unroll
-                                for (int j = 0; j < K; ++j) df_add_prod(acc[j], v, w[m][j]);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < K; ++j) sum[j] = make_float2(acc[j].hi, acc[j].lo);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < K; ++j) sum[j] = 0.0;
-                    if (!bad) {
-#pragma unroll
-                        for (int m = 0; m < kRsRT; ++m) {
-                            const int a = r + NR * m;
-                            if (a < rows) {
-                                const double v = (double)tile[a * K + i];
-#pragma unroll
-                                for (int j = 0; j < K; ++j) sum[j] = fma(v, (double)w[m][j], sum[j]);
-                            }
+                            for (int j = 0; j < K; ++j) sum[j] = fma(v, (double)w[m][j], sum[j]);
                         }
                     }
                 }
@@ -897,6 +882,156 @@ __global__ void __launch_bounds__(kRsCons + 64, sizeof(T) == 4 ? 2 : 1)
             }
             __syncwarp();
             if (lane == 0) bar_arrive(pfull0 + 8u * sr.s);
+        }
+    }
+}
+
+// hi + lo += a b for two independent pairs, products exact: t = fl(hi + p), p = fl(ab), and the two-sum's remainder with
+// ab in the place of p in its last difference: nb = -(t - hi), d = t + nb, (hi - d) + (ab + nb), where hi - d and p + nb are
+// exact and ab + nb, which is p + nb and the product's own rounding error together, is one fused multiply-add.  Eight packed
+// operations instead of ten; the remainder is within 2^-24 of itself either way.  (p itself cannot go: with t = fl(hi + ab)
+// a cancellation leaves t - hi and t + nb inexact.)
+// nz is -0, known only at run time: the product as fl(ab + nz).  A plain product is merged with the addition that follows
+// it into one fused multiply-add, by the assembler too where both are written as explicitly rounded f32x2 instructions
+// (measured: 2^-37 instead of 2^-48 of the sum under cancellation).
+__device__ __forceinline__ void df_fma2(float2 &hi, float2 &lo, float2 a, float2 b, float2 nz)
+{
+    const float2 m = make_float2(-1.0f, -1.0f);
+    const float2 t = __fadd2_rn(hi, __ffma2_rn(a, b, nz));
+    const float2 nb = __ffma2_rn(t, m, hi), d = __fadd2_rn(t, nb);
+    const float2 e = __fadd2_rn(__ffma2_rn(d, m, hi), __ffma2_rn(a, b, nb));
+    lo = __fadd2_rn(lo, e);
+    hi = t;
+}
+
+// V_b^T W for FP32 blocks with exact products (partial layout as rs_dots).
+// Block by block: a CTA streams the tiles b of V and W of all its chunks in
+// pairs through one ring, so that a block's sums stay in registers
+// (double-float, thread (r, i): V column i, rows r + (256 / K) m) over all of
+// them and lanes and warps are combined once per block instead of once per
+// tile; W comes from L2 from the second block on.  Bound by FP32 issue, 8
+// operations per product: 48Cr k = 8, 24 blocks 1.97 ms -> 0.90 ms (HBM floor
+// 0.23 ms).
+constexpr int kRxS = 5;   // ring stages of two tiles: 80 KB, two CTAs on an SM
+
+template <int K>
+__host__ __device__ constexpr size_t rx_smem()
+{
+    return 128 + (size_t)kRxS * 2 * kRsCE * 4 + 2 * (size_t)(kRsCons / 32) * K * K * sizeof(float2);
+}
+
+template <int K>
+__global__ void __launch_bounds__(kRsCons + 32, 2)
+    rs_dots_x(const float *__restrict__ V, int64_t bstride, int nb, const float *__restrict__ W, int64_t nel,
+              float2 *__restrict__ partial, const int *__restrict__ nb_iter, int *err, float minus_zero)
+{
+    using namespace tma;
+    using R = RsRed<float>;
+    constexpr int NR = kRsCons / K, NCW = kRsCons / 32;
+    const float2 nz = make_float2(minus_zero, minus_zero);
+    if (nb_iter) nb = *nb_iter + 1;   // graph replay: blocks 0..n of iteration n
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem);   // full[S], empty[S]
+    float *ring = reinterpret_cast<float *>(smem + 128);
+    float2 *red = reinterpret_cast<float2 *>(ring + (size_t)kRxS * 2 * kRsCE);   // [2][warps][K * K]
+    const uint32_t full0 = su32(bars), empty0 = su32(bars + kRxS);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int s = 0; s < kRxS; ++s) {
+            bar_init(full0 + 8u * s, 1);
+            bar_init(empty0 + 8u * s, NCW);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const int64_t nch = (nel + kRsCE - 1) / kRsCE;
+    RsRing<kRxS> q;
+    if (warp == NCW) {   // producer
+        if (lane != 0) return;
+        for (int b = 0; b < nb; ++b)
+            for (int64_t ch = blockIdx.x; ch < nch; ch += gridDim.x, q.next()) {
+                const int64_t e0 = ch * kRsCE;
+                const uint32_t bytes = (uint32_t)((min((int64_t)kRsCE, nel - e0) * 4 + 15) / 16 * 16);
+                if (q.uses >= kRxS && bar_wait(empty0 + 8u * q.s, q.ph ^ 1u)) {
+                    atomicExch(err, BS_ETIMEOUT);
+                    drain_ring(full0, kRxS, q.uses);
+                    return;
+                }
+                float *t = ring + (size_t)q.s * 2 * kRsCE;
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                bar_expect_tx(full0 + 8u * q.s, 2 * bytes);
+                bulk_copy(su32(t), V + (int64_t)b * bstride + e0, bytes, full0 + 8u * q.s);
+                bulk_copy(su32(t + kRsCE), W + e0, bytes, full0 + 8u * q.s);
+            }
+        return;
+    }
+    const int i = tid % K, r = tid / K;
+    bool bad = false;
+    for (int b = 0; b < nb; ++b) {
+        constexpr int NP = K == 1 ? 1 : K / 2;   // pairs of sums: columns 2q, 2q + 1 (K = 1: even and odd rows)
+        float2 hi[NP], lo[NP];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) hi[p] = lo[p] = make_float2(0.f, 0.f);
+        for (int64_t ch = blockIdx.x; ch < nch; ch += gridDim.x, q.next()) {
+            if (!bad && __any_sync(0xffffffffu, bar_wait(full0 + 8u * q.s, q.ph))) {
+                bad = true;
+                if (lane == 0) atomicExch(err, BS_ETIMEOUT);
+            }
+            const int rows = (int)(min((int64_t)kRsCE, nel - ch * kRsCE) / K);
+            const float *tv = ring + (size_t)q.s * 2 * kRsCE, *tw = tv + kRsCE;
+            if (!bad) {
+                if constexpr (K == 1) {
+#pragma unroll
+                    for (int m = 0; m < kRsRT; m += 2) {
+                        const int a = r + NR * m, c = a + NR;
+                        const float2 v = make_float2(a < rows ? tv[a] : 0.f, c < rows ? tv[c] : 0.f);
+                        const float2 w = make_float2(a < rows ? tw[a] : 0.f, c < rows ? tw[c] : 0.f);
+                        df_fma2(hi[0], lo[0], v, w, nz);
+                    }
+                } else {
+#pragma unroll
+                    for (int m = 0; m < kRsRT; ++m) {
+                        const int a = r + NR * m;
+                        if (a < rows) {
+                            const float v = tv[a * K + i];
+                            float w[K];
+                            ldrow<float, K>(tw + a * K, w);
+#pragma unroll
+                            for (int p = 0; p < NP; ++p)
+                                df_fma2(hi[p], lo[p], make_float2(v, v), make_float2(w[2 * p], w[2 * p + 1]), nz);
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) bar_arrive(empty0 + 8u * q.s);
+        }
+        // the warp's lanes of one column i, then the warps in order
+        float2 sum[K];
+        if constexpr (K == 1) {
+            sum[0] = R::add(make_float2(hi[0].x, lo[0].x), make_float2(hi[0].y, lo[0].y));
+        } else {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                sum[2 * p] = make_float2(hi[p].x, lo[p].x);
+                sum[2 * p + 1] = make_float2(hi[p].y, lo[p].y);
+            }
+        }
+#pragma unroll
+        for (int o = K; o < 32; o <<= 1)
+#pragma unroll
+            for (int j = 0; j < K; ++j) sum[j] = R::add(sum[j], R::shfl(sum[j], o));
+        float2 *rb = red + (size_t)(b & 1) * NCW * K * K;
+        if (lane < K) {
+#pragma unroll
+            for (int j = 0; j < K; ++j) rb[((size_t)warp * K + i) * K + j] = sum[j];
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kRsCons) : "memory");   // the consumer warps only
+        if (tid < K * K) {
+            float2 t = rb[tid];
+#pragma unroll
+            for (int w2 = 1; w2 < NCW; ++w2) t = R::add(t, rb[(size_t)w2 * K * K + tid]);
+            partial[((int64_t)blockIdx.x * nb + b) * K * K + tid] = t;
         }
     }
 }
@@ -1312,7 +1447,23 @@ void dots(LState &L, const T *V, int nb, const T *W, double *out, const int *nb_
             return;
         }
     }
-    if (rs_applies<T, K>(L, V, W)) {
+    if constexpr (EXACT && std::is_same<T, float>::value) {
+        if (rs_applies<T, K>(L, V, W)) {
+            constexpr size_t smem = rx_smem<K>();
+            static unsigned long long attr = 0;   // per instantiation: devices already configured
+            int dev = 0;
+            cudaGetDevice(&dev);
+            if (dev < 64 && !(attr >> dev & 1ull)) {
+                cudaFuncSetAttribute(rs_dots_x<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                attr |= 1ull << dev;
+            }
+            rs_dots_x<K><<<L.ncta, kRsCons + 32, smem, L.s>>>(V, L.bstride, nb, W, L.dim * K, reinterpret_cast<float2 *>(L.partial),
+                                                              nb_iter, L.err, -0.0f);
+            reduce_parts<float2>(reinterpret_cast<const float2 *>(L.partial), L.ncta, n, nb * K * K, out, nb_iter, out_iter,
+                                 K * K, L.s);
+            return;
+        }
+    } else if (rs_applies<T, K>(L, V, W)) {
         using Sv = typename RsRed<T>::S;
         constexpr int S = rs_stages<T>();
         const size_t acc = (size_t)(nb_iter ? nb_max : nb) * K * K * sizeof(Sv);
