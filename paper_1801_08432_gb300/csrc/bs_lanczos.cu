@@ -1127,6 +1127,8 @@ __global__ void __launch_bounds__(kRwCons + 32, 1)
     const int64_t rpc = (dim + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = (int64_t)blockIdx.x * rpc, r1 = min(dim, r0 + rpc);
     float2 *part = partial + (int64_t)blockIdx.x * nb * K * K;
+    // grid.y CTAs share the rows' blocks (small bases: too few rows for the chip)
+    const int b0 = (int)((int64_t)nb * blockIdx.y / gridDim.y), b1 = (int)((int64_t)nb * (blockIdx.y + 1) / gridDim.y);
     if (warp == NCW) {   // producer
         if (lane != 0) return;
         int64_t tiles = 0, wcopies = 0;
@@ -1136,10 +1138,10 @@ __global__ void __launch_bounds__(kRwCons + 32, 1)
             const int64_t pr = min((int64_t)PR, r1 - p0);
             const int nt = (int)((pr + TR - 1) / TR);
             int s = (int)(tiles % kRwS);
-            for (int b = 0; ok && b < nb; ++b)
+            for (int b = b0; ok && b < b1; ++b)
                 for (int t = 0; t < nt; ++t, ++tiles, s = s + 1 == kRwS ? 0 : s + 1) {
                     const uint32_t bytes = (uint32_t)(min((int64_t)TR, pr - (int64_t)t * TR) * RB);
-                    if (b == 0) {   // W slot t: free once the previous piece's last block used it
+                    if (b == b0) {   // W slot t: free once the previous piece's last block used it
                         if (piece > 0 && bar_wait(wempty0 + 8u * t, (uint32_t)(piece - 1) & 1u)) { ok = false; break; }
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         bar_expect_tx(wfull0 + 8u * t, bytes);
@@ -1177,7 +1179,7 @@ __global__ void __launch_bounds__(kRwCons + 32, 1)
     for (int64_t p0 = r0; p0 < r1; p0 += PR, ++piece) {
         const int64_t pr = min((int64_t)PR, r1 - p0);
         const int nt = (int)((pr + TR - 1) / TR);
-        for (int b = 0; b < nb; ++b, ++nred) {
+        for (int b = b0; b < b1; ++b, ++nred) {
             // this block's running partial, read now so that the load is done by the end of the piece
             float2 prev = make_float2(0.f, 0.f);
             if (piece > 0 && tid < K * K) prev = part[(int64_t)b * K * K + tid];
@@ -1188,7 +1190,7 @@ __global__ void __launch_bounds__(kRwCons + 32, 1)
 #pragma unroll
             for (int t = 0; t < kRwWT; ++t) {   // unrolled: slot addresses and barriers are constants
                 if (t >= nt) break;
-                if (b == 0 && !bad && __any_sync(0xffffffffu, bar_wait(wfull0 + 8u * t, (uint32_t)piece & 1u))) {
+                if (b == b0 && !bad && __any_sync(0xffffffffu, bar_wait(wfull0 + 8u * t, (uint32_t)piece & 1u))) {
                     bad = true;
                     if (lane == 0) atomicExch(err, BS_ETIMEOUT);
                 }
@@ -1235,7 +1237,7 @@ __global__ void __launch_bounds__(kRwCons + 32, 1)
                 __syncwarp();
                 if (lane == 0) {
                     bar_arrive(empty0 + 8u * s);
-                    if (b == nb - 1) bar_arrive(wempty0 + 8u * t);
+                    if (b == b1 - 1) bar_arrive(wempty0 + 8u * t);
                 }
                 if (++s == kRwS) {
                     s = 0;
@@ -1297,7 +1299,7 @@ __global__ void __launch_bounds__(kRwCons + 32, 1)
         }
     }
     if (r0 >= r1) {   // no rows for this CTA: its partials are zero
-        for (int e = tid; e < nb * K * K; e += kRwCons) part[e] = make_float2(0.f, 0.f);
+        for (int e = b0 * K * K + tid; e < b1 * K * K; e += kRwCons) part[e] = make_float2(0.f, 0.f);
     }
 }
 
@@ -1308,21 +1310,21 @@ __global__ void __launch_bounds__(kRwCons + 32, 1)
 // warp-uniform broadcasts, each C_b row serving all of its rows (the C reads
 // bound shared memory at one row per thread).  FP32 pairs of
 // columns go through two-wide FMAs, each component rounded as fmaf would.
-template <typename T, int K, int S>
+template <typename T, int K, int S, int CE>
 __global__ void __launch_bounds__(kRsCons + 32) rs_update(const T *__restrict__ V, int64_t bstride, int nb,
                                                           const double *__restrict__ C, T *__restrict__ W,
                                                           int64_t nel, const int *__restrict__ nb_iter,
                                                           const int *__restrict__ c_iter, int *err)
 {
     using namespace tma;
-    constexpr int RU = kRsCEU / K / kRsCons;   // rows per thread per tile
+    constexpr int RU = CE / K / kRsCons;   // rows per thread per tile
     constexpr bool PACKED = std::is_same<T, float>::value && K >= 2;
     if (nb_iter) nb = *nb_iter + 1;
     if (c_iter) C += (int64_t)(*c_iter) * K * K;
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
     T *ring = reinterpret_cast<T *>(smem + 128);
-    T *Cs = ring + (size_t)S * kRsCEU;   // [nb][i][j]
+    T *Cs = ring + (size_t)S * CE;   // [nb][i][j]
     const uint32_t full0 = su32(bars), empty0 = su32(bars + S);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
@@ -1335,22 +1337,22 @@ __global__ void __launch_bounds__(kRsCons + 32) rs_update(const T *__restrict__ 
     for (int e = tid; e < nb * K * K; e += blockDim.x) Cs[e] = (T)C[e];
     __syncthreads();
     if (warp == kRsCons / 32) {
-        if (lane == 0 && !rs_produce<T, S, kRsCEU>(V, bstride, nb, W, nel, ring, full0, empty0)) atomicExch(err, BS_ETIMEOUT);
+        if (lane == 0 && !rs_produce<T, S, CE>(V, bstride, nb, W, nel, ring, full0, empty0)) atomicExch(err, BS_ETIMEOUT);
         return;
     }
-    const int64_t nch = (nel + kRsCEU - 1) / kRsCEU;
+    const int64_t nch = (nel + CE - 1) / CE;
     RsRing<S> q;
     bool bad = false;
     for (int64_t ch = blockIdx.x; ch < nch; ch += gridDim.x) {
-        const int64_t e0 = ch * kRsCEU;
-        const int rows = (int)(min((int64_t)kRsCEU, nel - e0) / K);
+        const int64_t e0 = ch * CE;
+        const int rows = (int)(min((int64_t)CE, nel - e0) / K);
         T w[RU][K];
         for (int b = -1; b < nb; ++b, q.next()) {
             if (!bad && __any_sync(0xffffffffu, bar_wait(full0 + 8u * q.s, q.ph))) {
                 bad = true;
                 if (lane == 0) atomicExch(err, BS_ETIMEOUT);
             }
-            const T *tile = ring + (size_t)q.s * kRsCEU;
+            const T *tile = ring + (size_t)q.s * CE;
             if (b < 0) {
 #pragma unroll
                 for (int m = 0; m < RU; ++m) {
@@ -1439,8 +1441,12 @@ void dots(LState &L, const T *V, int nb, const T *W, double *out, const int *nb_
                 cudaFuncSetAttribute(rs_dots_w<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 attr |= 1ull << dev;
             }
-            const int g = std::min(nsm, L.ncta);   // one CTA per SM; the partials hold L.ncta
-            rs_dots_w<K><<<g, kRwCons + 32, smem, L.s>>>(V, L.bstride, nb, W, L.dim, reinterpret_cast<float2 *>(L.partial),
+            // one CTA per SM; the partials hold L.ncta.  Ranges of at least a tile (a thread of a shorter one has
+            // no row of its own), the SMs left over share the blocks: sd 4p4n k = 4, 22 -> 8 us a pass
+            constexpr int64_t TR = (int64_t)(kRwTile / (K * 4) / kRwCons) * kRwCons;
+            const int g = (int)std::min<int64_t>(std::min(nsm, L.ncta), (L.dim + TR - 1) / TR);
+            const int gy = std::max(1, std::min(nb_iter ? nb_max : nb, std::min(nsm, L.ncta) / g));
+            rs_dots_w<K><<<dim3((unsigned)g, (unsigned)gy), kRwCons + 32, smem, L.s>>>(V, L.bstride, nb, W, L.dim, reinterpret_cast<float2 *>(L.partial),
                                                         nb_iter, L.err);
             reduce_parts<float2>(reinterpret_cast<const float2 *>(L.partial), g, n, nb * K * K, out, nb_iter, out_iter,
                                  K * K, L.s);
@@ -1490,6 +1496,20 @@ void dots(LState &L, const T *V, int nb, const T *W, double *out, const int *nb_
     reduce_parts<double>(L.partial, L.ncta, n, nb * K * K, out, nb_iter, out_iter, K * K, L.s);
 }
 
+template <typename T, int K, int S, int CE>
+void launch_update(LState &L, const T *V, int nb, const double *C, T *W, const int *nb_iter, const int *c_iter, size_t csm)
+{
+    static unsigned long long attr = 0;   // per instantiation: devices already configured
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 64 && !(attr >> dev & 1ull)) {
+        cudaFuncSetAttribute(rs_update<T, K, S, CE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+        attr |= 1ull << dev;
+    }
+    rs_update<T, K, S, CE><<<L.ncta, kRsCons + 32, 128 + (size_t)S * CE * sizeof(T) + csm, L.s>>>(V, L.bstride, nb, C, W, L.dim * K,
+                                                                                                nb_iter, c_iter, L.err);
+}
+
 template <typename T, int K>
 void update(LState &L, const T *V, int nb, const double *C, T *W, const int *nb_iter = nullptr,
             const int *c_iter = nullptr, int nb_max = 0)
@@ -1499,14 +1519,10 @@ void update(LState &L, const T *V, int nb, const double *C, T *W, const int *nb_
     constexpr int S = sizeof(T) == 4 ? 3 : 2;   // 16 KB (FP32) or 32 KB (FP64) tiles
     const size_t rsm = 128 + (size_t)S * kRsCEU * sizeof(T) + csm;
     if (rs_applies<T, K>(L, V, W) && rsm <= 112 * 1024) {
-        static unsigned long long attr = 0;   // per instantiation: devices already configured
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 64 && !(attr >> dev & 1ull)) {
-            cudaFuncSetAttribute(rs_update<T, K, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
-            attr |= 1ull << dev;
-        }
-        rs_update<T, K, S><<<L.ncta, kRsCons + 32, rsm, L.s>>>(V, L.bstride, nb, C, W, L.dim * K, nb_iter, c_iter, L.err);
+        // tiles of one row per thread where the larger ones (more rows per read of C) leave CTAs without any:
+        // sd 4p4n k = 4, 28 tiles for 304 CTAs, 9.9 -> 8.7 us a pass
+        if (L.dim * K < (int64_t)kRsCEU * L.ncta) launch_update<T, K, S, kRsCons * K>(L, V, nb, C, W, nb_iter, c_iter, csm);
+        else launch_update<T, K, S, kRsCEU>(L, V, nb, C, W, nb_iter, c_iter, csm);
         return;
     }
     blk_update<T, K><<<L.ncta, 256, csm, L.s>>>(V, L.bstride, nb, C, W, L.dim, nb_iter, c_iter);
