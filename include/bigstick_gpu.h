@@ -409,7 +409,7 @@ int bs_debug_eigh_banded(int n, int bw, const double *A, int nval, double *w, do
  * neutron-list buffers; 17, 18, 19: 227 KB, two list buffers; 20: 227 KB,
  * three list buffers; 16: the pn term by pairs of a (Z-1)-proton and an
  * (N-1)-neutron core, a dense product per group of neutron cores, for every
- * k and for W-truncated bases too); in 11, 12, 17
+ * k); in 11, 12, 17
  * the pipelined kernel computes the like-particle terms into one more (17:
  * the first pipelined variant that fits, for neutron sectors wider than 576
  * columns); in 13..16 and 18..20 a second persistent kernel computes the pp
@@ -417,8 +417,8 @@ int bs_debug_eigh_banded(int n, int bw, const double *A, int nval, double *w, do
  * (Z-2)-proton core into C(Z,2) more and a row-tile kernel (4 rows per CTA,
  * 2 in 19 and 20, column tiles of 576 for wider sectors; 18: the first pipelined
  * variant that fits) the nn term and the proton single-particle energies
- * into one more (16 with k = 1, 2 or a W-truncated basis: panels of x in
- * shared memory for both like-particle terms, which add the partial vectors);
+ * into one more (16 with k = 1, 2: panels of x in shared memory for
+ * both like-particle terms, which add the partial vectors);
  * a last kernel
  * sums the partial vectors in a fixed order (workspace: up to
  * (Z + C(Z,2) + 1) x dim x k floats, allocated on first use, or by

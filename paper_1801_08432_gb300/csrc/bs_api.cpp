@@ -290,22 +290,20 @@ int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std
         (R == 2 ? D.nnntasks2 : D.nnntasks4) = (int)nt.size();
         if ((rc = put(D, dst, nt.data(), nt.size(), err))) return rc;
     }
-    for (int spc = 0; spc < 2; ++spc) {   // like-particle panels
+    for (int spc = 0; spc < 2 && T.pair.on; ++spc) {   // like-particle panels
         Device::LikeDev &q = D.like[spc];
-        LikePanels O;
-        build_like_panels(B, spc, 8, O);
-        q.max_n = O.max_n;
-        q.pw = like_panel_width(O.max_n);
+        std::vector<LikePanel> O;
+        build_like_panels(B, spc, 32, O, q.max_n);
+        q.pw = like_panel_width(q.max_n);
         if (!q.pw) continue;
         LikeLists L;
-        build_like_lists(B, spc, spc ? T.nn : T.pp, spc ? T.nnx : T.ppx, L);
+        build_like_lists(spc ? T.nn : T.pp, L);
         if ((rc = put(D, q.ptr, L.ptr.data(), L.ptr.size(), err))) return rc;
         if ((rc = put(D, q.ent, L.ent.data(), L.ent.size(), err))) return rc;
-        if ((rc = put(D, q.pieces, O.pieces.data(), O.pieces.size(), err))) return rc;
-        for (int v = 0; v < 4; ++v) {
-            build_like_panels(B, spc, q.pw >> v, O);
-            q.npanels[v] = (int)O.panels.size();
-            if ((rc = put(D, q.panels[v], O.panels.data(), O.panels.size(), err))) return rc;
+        for (int v = 0; v < 2; ++v) {
+            build_like_panels(B, spc, q.pw >> v, O, q.max_n);
+            q.npanels[v] = (int)O.size();
+            if ((rc = put(D, q.panels[v], O.data(), O.size(), err))) return rc;
         }
     }
     if (T.pair.on) {   // pair-core pn kernel

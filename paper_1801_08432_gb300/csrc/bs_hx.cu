@@ -19,6 +19,8 @@
 // and the pn links already join any pair of blocks.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "bs_internal.h"
 
 namespace bs {
@@ -85,106 +87,131 @@ struct HxArgs {
     const int32_t *ppx_src, *nnx_src;
 };
 
-template <typename T, int K>
-__global__ void __launch_bounds__(128) hx_fused_kernel(HxArgs A, const T *__restrict__ pp_coef,
-                                                       const T *__restrict__ nn_coef, const T *__restrict__ wpn,
-                                                       const T *__restrict__ ppx_coef, const T *__restrict__ nnx_coef,
-                                                       const T *__restrict__ x, T *__restrict__ y)
+// A CTA's warps beyond the tile's columns form further groups (G in all): group
+// g takes every G-th like-particle entry and every G-th pn link, and the
+// groups' sums meet in shared memory, in the order of the groups.  A thread's
+// chain of dependent loads (list pointer, entry, element) is what bounds the
+// kernel on small bases and narrow sectors, where the extra warps cost
+// nothing.
+template <typename T, int K, int NT>
+__global__ void __launch_bounds__(NT) hx_fused_kernel(HxArgs A, const T *__restrict__ pp_coef,
+                                                      const T *__restrict__ nn_coef, const T *__restrict__ wpn,
+                                                      const T *__restrict__ ppx_coef, const T *__restrict__ nnx_coef,
+                                                      const T *__restrict__ x, T *__restrict__ y)
 {
+    __shared__ __align__(16) T part[NT > 128 ? NT - 32 : 96][K];
     const DevTask t = A.tasks[blockIdx.x];
     const DevBlock D = A.blocks[t.block];
-    const int col = t.col0 + (int)threadIdx.x;
-    if (col >= D.nN) return;
+    const int cw = (min(128, D.nN - t.col0) + 31) / 32;          // warps of a group
+    const int G = NT / 32 / cw, g = (int)(threadIdx.x >> 5) / cw;
+    const int lc = (int)threadIdx.x - g * cw * 32;               // column in the tile
+    const int col = t.col0 + lc;
+    const bool live = g < G && col < D.nN;
     T acc[K];
 #pragma unroll
     for (int c = 0; c < K; ++c) acc[c] = T(0);
     T xv[K];
-
-    // pp (same block): rows ip of x, column col
-    {
-        const int g = D.p_start + t.row;
-        const int64_t e1 = A.pp_ptr[g + 1];
-        const T *xc = x + (D.off + col) * K;
-        for (int64_t e = A.pp_ptr[g]; e < e1; ++e) {
-            const T c = pp_coef[e];
-            ldk<T, K>(xc + (int64_t)A.pp_src[e] * D.nN * K, xv);
-#pragma unroll
-            for (int q = 0; q < K; ++q) acc[q] = fma(c, xv[q], acc[q]);
-        }
-    }
-    // nn (same block): row ip', columns jn
-    {
-        const int g = D.n_start + col;
-        const int64_t e1 = A.nn_ptr[g + 1];
-        const T *xr = x + (D.off + (int64_t)t.row * D.nN) * K;
-        for (int64_t e = A.nn_ptr[g]; e < e1; ++e) {
-            const T c = nn_coef[e];
-            ldk<T, K>(xr + (int64_t)A.nn_src[e] * K, xv);
-#pragma unroll
-            for (int q = 0; q < K; ++q) acc[q] = fma(c, xv[q], acc[q]);
-        }
-    }
-    // like-particle moves from other blocks (W-truncated bases): pp moves from
-    // the block of another proton sector with this neutron sector (same
-    // column), nn moves from the block of another neutron sector with this
-    // proton sector (same row)
-    for (int L = D.llink_begin; L < D.llink_end; ++L) {
-        const DevLLink lk = A.llinks[L];
-        const DevBlock S = A.blocks[lk.src_block];
-        if (lk.species == 0) {
-            const int64_t e1 = A.ppx_ptr[lk.ptr_off + t.row + 1];
-            const T *xc = x + (S.off + col) * K;
-            for (int64_t e = A.ppx_ptr[lk.ptr_off + t.row]; e < e1; ++e) {
-                const T c = ppx_coef[e];
-                ldk<T, K>(xc + (int64_t)A.ppx_src[e] * S.nN * K, xv);
-#pragma unroll
-                for (int q = 0; q < K; ++q) acc[q] = fma(c, xv[q], acc[q]);
-            }
-        } else {
-            const int64_t e1 = A.nnx_ptr[lk.ptr_off + col + 1];
-            const T *xr = x + (S.off + (int64_t)t.row * S.nN) * K;
-            for (int64_t e = A.nnx_ptr[lk.ptr_off + col]; e < e1; ++e) {
-                const T c = nnx_coef[e];
-                ldk<T, K>(xr + (int64_t)A.nnx_src[e] * K, xv);
+    if (live) {
+        // pp (same block): rows ip of x, column col
+        {
+            const int gr = D.p_start + t.row;
+            const int64_t e1 = A.pp_ptr[gr + 1];
+            const T *xc = x + (D.off + col) * K;
+#pragma unroll 4
+            for (int64_t e = A.pp_ptr[gr] + g; e < e1; e += G) {
+                const T c = pp_coef[e];
+                ldk<T, K>(xc + (int64_t)A.pp_src[e] * D.nN * K, xv);
 #pragma unroll
                 for (int q = 0; q < K; ++q) acc[q] = fma(c, xv[q], acc[q]);
             }
         }
-    }
-    // pn: proton one-body jump x neutron one-body jump, per linked source block
-    for (int L = D.link_begin; L < D.link_end; ++L) {
-        const DevLink lk = A.links[L];
-        const int64_t pb = A.p1_ptr[lk.p_ptr_off + t.row], pe = A.p1_ptr[lk.p_ptr_off + t.row + 1];
-        if (pb == pe) continue;
-        const int64_t nb0 = A.n1_ptr[lk.n_ptr_off + col], ne0 = A.n1_ptr[lk.n_ptr_off + col + 1];
-        if (nb0 == ne0) continue;
-        const DevBlock S = A.blocks[lk.src_block];
-        const T *W = wpn + lk.w_off;
-        for (int64_t u = pb; u < pe; ++u) {
-            const uint32_t ep = A.p1_ent[u];
-            const T *xr = x + (S.off + (int64_t)(ep & 0xFFFFu) * S.nN) * K;
-            const T *Wa = W + (int64_t)((ep >> 16) & 0x7FFFu) * lk.nb;
-            T part[K];
+        // nn (same block): row ip', columns jn
+        {
+            const int gn = D.n_start + col;
+            const int64_t e1 = A.nn_ptr[gn + 1];
+            const T *xr = x + (D.off + (int64_t)t.row * D.nN) * K;
+#pragma unroll 4
+            for (int64_t e = A.nn_ptr[gn] + g; e < e1; e += G) {
+                const T c = nn_coef[e];
+                ldk<T, K>(xr + (int64_t)A.nn_src[e] * K, xv);
 #pragma unroll
-            for (int q = 0; q < K; ++q) part[q] = T(0);
-            for (int64_t v = nb0; v < ne0; ++v) {
-                const uint32_t en = A.n1_ent[v];
-                T w = __ldg(Wa + ((en >> 16) & 0x7FFFu));
-                if (en >> 31) w = -w;
-                ldk<T, K>(xr + (int64_t)(en & 0xFFFFu) * K, xv);
-#pragma unroll
-                for (int q = 0; q < K; ++q) part[q] = fma(w, xv[q], part[q]);
+                for (int q = 0; q < K; ++q) acc[q] = fma(c, xv[q], acc[q]);
             }
-            if (ep >> 31) {
+        }
+        // like-particle moves from other blocks (W-truncated bases): pp moves from
+        // the block of another proton sector with this neutron sector (same
+        // column), nn moves from the block of another neutron sector with this
+        // proton sector (same row)
+        for (int L = D.llink_begin + g; L < D.llink_end; L += G) {
+            const DevLLink lk = A.llinks[L];
+            const DevBlock S = A.blocks[lk.src_block];
+            if (lk.species == 0) {
+                const int64_t e1 = A.ppx_ptr[lk.ptr_off + t.row + 1];
+                const T *xc = x + (S.off + col) * K;
+                for (int64_t e = A.ppx_ptr[lk.ptr_off + t.row]; e < e1; ++e) {
+                    const T c = ppx_coef[e];
+                    ldk<T, K>(xc + (int64_t)A.ppx_src[e] * S.nN * K, xv);
 #pragma unroll
-                for (int q = 0; q < K; ++q) acc[q] -= part[q];
+                    for (int q = 0; q < K; ++q) acc[q] = fma(c, xv[q], acc[q]);
+                }
             } else {
+                const int64_t e1 = A.nnx_ptr[lk.ptr_off + col + 1];
+                const T *xr = x + (S.off + (int64_t)t.row * S.nN) * K;
+                for (int64_t e = A.nnx_ptr[lk.ptr_off + col]; e < e1; ++e) {
+                    const T c = nnx_coef[e];
+                    ldk<T, K>(xr + (int64_t)A.nnx_src[e] * K, xv);
 #pragma unroll
-                for (int q = 0; q < K; ++q) acc[q] += part[q];
+                    for (int q = 0; q < K; ++q) acc[q] = fma(c, xv[q], acc[q]);
+                }
+            }
+        }
+        // pn: proton one-body jump x neutron one-body jump, per linked source block
+        for (int L = D.link_begin + g; L < D.link_end; L += G) {
+            const DevLink lk = A.links[L];
+            const int64_t pb = A.p1_ptr[lk.p_ptr_off + t.row], pe = A.p1_ptr[lk.p_ptr_off + t.row + 1];
+            const int64_t nb0 = A.n1_ptr[lk.n_ptr_off + col], ne0 = A.n1_ptr[lk.n_ptr_off + col + 1];
+            if (pb == pe || nb0 == ne0) continue;
+            const DevBlock S = A.blocks[lk.src_block];
+            const T *W = wpn + lk.w_off;
+            for (int64_t u = pb; u < pe; ++u) {
+                const uint32_t ep = A.p1_ent[u];
+                const T *xr = x + (S.off + (int64_t)(ep & 0xFFFFu) * S.nN) * K;
+                const T *Wa = W + (int64_t)((ep >> 16) & 0x7FFFu) * lk.nb;
+                T part[K];
+#pragma unroll
+                for (int q = 0; q < K; ++q) part[q] = T(0);
+#pragma unroll 2
+                for (int64_t v = nb0; v < ne0; ++v) {
+                    const uint32_t en = A.n1_ent[v];
+                    T w = __ldg(Wa + ((en >> 16) & 0x7FFFu));
+                    if (en >> 31) w = -w;
+                    ldk<T, K>(xr + (int64_t)(en & 0xFFFFu) * K, xv);
+#pragma unroll
+                    for (int q = 0; q < K; ++q) part[q] = fma(w, xv[q], part[q]);
+                }
+                if (ep >> 31) {
+#pragma unroll
+                    for (int q = 0; q < K; ++q) acc[q] -= part[q];
+                } else {
+#pragma unroll
+                    for (int q = 0; q < K; ++q) acc[q] += part[q];
+                }
             }
         }
     }
-    stk<T, K>(y + (D.off + (int64_t)t.row * D.nN + col) * K, acc);
+    if (G > 1) {   // CTA-uniform
+        if (live && g > 0) {
+#pragma unroll
+            for (int q = 0; q < K; ++q) part[(g - 1) * cw * 32 + lc][q] = acc[q];
+        }
+        __syncthreads();
+        if (live && g == 0) {
+            for (int h = 1; h < G; ++h)
+#pragma unroll
+                for (int q = 0; q < K; ++q) acc[q] += part[(h - 1) * cw * 32 + lc][q];
+        }
+    }
+    if (live && g == 0) stk<T, K>(y + (D.off + (int64_t)t.row * D.nN + col) * K, acc);
 }
 
 template <typename T, int K>
@@ -192,7 +219,18 @@ cudaError_t launch(const Device &Dv, const DevCoefs<T> &C, const T *x, T *y, cud
 {
     HxArgs A{Dv.tasks, Dv.blocks, Dv.links, Dv.pp_ptr, Dv.nn_ptr, Dv.p1_ptr, Dv.n1_ptr,
              Dv.pp_src, Dv.nn_src, Dv.p1_ent, Dv.n1_ent, Dv.llinks, Dv.ppx_ptr, Dv.nnx_ptr, Dv.ppx_src, Dv.nnx_src};
-    hx_fused_kernel<T, K><<<Dv.ntasks, Dv.tile, 0, s>>>(A, C.pp_coef, C.nn_coef, C.wpn, C.ppx_coef, C.nnx_coef, x, y);
+    auto run = [&](auto nt) {
+        constexpr int NT = decltype(nt)::value;
+        hx_fused_kernel<T, K, NT><<<Dv.ntasks, NT, 0, s>>>(A, C.pp_coef, C.nn_coef, C.wpn, C.ppx_coef, C.nnx_coef, x, y);
+    };
+    // Threads by the number of CTAs: with few, more groups shorten each thread's chain of loads; with many, they only
+    // take registers.  us at 128 / 256 / 512 threads: sd 2p2n (66 CTAs) FP64 k = 1 17 / 15 / 16; sd 4p4n (495) FP32
+    // k = 4 51 / 37 / 34, k = 8 64 / 47 / 49, FP64 k = 8 297 / 254 / 293; pf 3p3n (2,200) k = 1 111 / 98 / 130,
+    // k = 4 126 / 154 / 152, k = 8 228 / 219 / 249; pf 4p3n (9,500) k = 1 398 / 413 / 585.
+    constexpr bool wide = K * sizeof(T) == 64;
+    if (Dv.ntasks < 1000 && !wide) run(std::integral_constant<int, 512>{});
+    else if (Dv.ntasks < 1000 || (Dv.ntasks < 2500 && (K == 1 || K == 8))) run(std::integral_constant<int, 256>{});
+    else run(std::integral_constant<int, 128>{});
     return cudaGetLastError();
 }
 
@@ -236,33 +274,35 @@ int launch_hx(const bs_ctx *c, const void *x, void *y, int k, bs_dtype dt, void 
     if (mode == 0 && e == cudaSuccess) {
         const int64_t dim = c->basis.dim;
         if (dt == BS_F64 || c->dev.trunc) {
-            // the first pipelined variant, else the first row variant, else the tiled kernel
-            e = launch_hx_pipe(c, x, y, k, dt, s, 0, used);
-            if (!used) mode = 2;
+            // the first pipelined variant, else the first row variant, else the tiled kernel; small bases the tiled
+            // kernel (FP64 k = 1, us, tiled / row: sd 2p2n 15 / 37, sd 4p4n 70 / 95, pf 2p3n 62 / 68, sd 5p6n 182 / 133)
+            if (dim < 50000) {
+                mode = 1;
+            } else {
+                e = launch_hx_pipe(c, x, y, k, dt, s, 0, used);
+                if (!used) mode = 2;
+            }
         } else {
             // FP32, not tuned.  Measured on this chip, us per product of k = 4 (k = 2) by the tiled / pipelined
             // (row) / core-grouped / pair-core kernels:
-            //   sd 4p4n 58 / 51 / 82 / 67 (47 / 71 / - / 56);  pf 3p3n 203 / 152 / 168 / 163 (161 / 179 / - / 109);
-            //   pf 4p3n 571 / 741 / 929 / 685 (449 / 762 / - / 353);  pf 4p4n 2847 / 2103 / 1232 / 1141 (2138 / 2236 / - / 725);
-            //   pf 6p2n (neutron sectors of 30) 985 / 5779 / 9782 / - (772 / 4947 / - / -);
+            //   sd 4p4n 34 / 51 / 82 / 67 (31 / 71 / - / 56);  pf 3p3n 126 / 152 / 168 / 163 (100 / 179 / - / 109);
+            //   pf 4p3n 512 / 741 / 929 / 685 (400 / 762 / - / 353);  pf 4p4n 2761 / 2103 / 1232 / 1141 (1820 / 2236 / - / 725);
+            //   pf 6p2n (neutron sectors of 30) 892 / 5779 / 9782 / - (743 / 4947 / - / -);
             // at k = 8 the core-grouped kernels lead from 100,000 states and sectors of 64 columns on.
             const int nN = c->dev.max_nN;
-            const bool small = dim < 100000, narrow = nN < 64;
-            if (!small && narrow) mode = 1;                            // the wide kernels give a thread a column
-            else if (k < 4) mode = small ? 2 : kPairMode;
-            else if (small) mode = 2 + R;                              // one CTA per row fills the chip
-            else if (k == 4 && nN < 256) mode = dim < 300000 ? 2 + R : 1;
-            else mode = k == 4 ? kPairMode : kCoreMode;
+            if (dim < 100000 || nN < 64) mode = 1;                     // (the wide kernels give a thread a column)
+            else if (k < 4) mode = kPairMode;
+            else if (k == 4) mode = nN < 256 ? 1 : kPairMode;
+            else mode = kCoreMode;
             if (mode == kPairMode || mode == kCoreMode) {
                 // a form that does not fit this basis: the next one
                 for (int m : {mode, (int)kCoreMode, 13})
                     if (e == cudaSuccess && !used) e = launch_hx_core(c, x, y, k, dt, s, m - 2 - R - pipe_variants(), used, t0, t1);
                 core_used = used;
-                if (!used) mode = 2 + R;
-            }
-            if (e == cudaSuccess && !used && mode == 2 + R) {
-                e = launch_hx_pipe(c, x, y, k, dt, s, 0, used);
-                if (!used) mode = 2;
+                if (!used) {
+                    e = e == cudaSuccess ? launch_hx_pipe(c, x, y, k, dt, s, 0, used) : e;
+                    if (!used) mode = 2;
+                }
             }
         }
     }

@@ -1003,12 +1003,12 @@ size_t pair_bytes(const bs_ctx *c, int k)
     return (size_t)c->basis.Z * (size_t)c->basis.dim * (size_t)k * sizeof(float);
 }
 
-// The pair-core kernel without the core-grouped like-particle kernels: its Z
+// k = 1, 2: the pair-core kernel without the core-grouped like-particle kernels: its Z
 // partial vectors go to the like-particle panels.
 bool pair_applies(const bs_ctx *c, int k, bs_dtype dt)
 {
     bool fits = false;
-    return dt == BS_F32 && like_applies(c) && launch_hx_pair(c, nullptr, nullptr, k, nullptr, fits) == cudaSuccess && fits;
+    return dt == BS_F32 && k < 4 && like_applies(c) && launch_hx_pair(c, nullptr, nullptr, k, nullptr, fits) == cudaSuccess && fits;
 }
 
 bool core_applies(const bs_ctx *c, int k, bs_dtype dt)
@@ -1047,7 +1047,12 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
     used = false;
     if (v < 0 || v >= kNumCore) return cudaSuccess;
     const bool pair = kCoreVariants[v].pair, core = core_applies(c, k, dt);
-    if (!(core && !pair) && !(pair && pair_applies(c, k, dt))) return cudaSuccess;
+    if (!core && !(pair && pair_applies(c, k, dt))) return cudaSuccess;
+    if (core && pair) {
+        bool ok = false;
+        const cudaError_t pe = launch_hx_pair(c, nullptr, nullptr, k, s, ok);
+        if (pe != cudaSuccess || !ok) return pe;
+    }
     if (c->core_part_bytes < (core ? part_bytes(c, k) : pair_bytes(c, k))) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         cudaError_t e = cudaStreamIsCapturing(s, &cap);

@@ -1,10 +1,10 @@
-// Like-particle terms of y = H x, k = 1, 2, 4, 8, plain and W-truncated bases
-// (sm_103a), as two sparse products with uniform lists:
+// Like-particle terms of y = H x for k = 1, 2 (sm_103a), as two sparse
+// products with uniform lists:
 //   nn:  y[r, q]  = sum_s Hnn[q, s] x[r, s]   over the neutron SDs s,
 //   pp:  y[r, q] += sum_s Hpp[r, s] x[s, q]   over the proton SDs s, plus the
 //                                              partial vectors of the pn term.
 // One species' matrix is the same for every SD of the other, so a CTA stages
-// a panel of x in shared memory, all SDs of one (2M, parity) of the acting
+// a panel of x in shared memory, all SDs of one sector of the acting
 // species by 256 bytes of the other's (64 / K SDs of K components, 32 / K
 // for more than 840 SDs), and a warp owns a whole output row of the panel:
 // its 32 lanes hold the row's columns, so the list entry (source, coefficient)
@@ -14,10 +14,8 @@
 // Against lists per lane (a lane gathers its own column's sources) this reads
 // no padding and no conflicts, and an entry costs 8 bytes per 64
 // multiply-adds instead of 8 bytes per lane: 0.19 ms for both terms at pf
-// 4p4n k = 2 against 0.60 ms by the tiled kernel without its pn term.  The acting species' SDs of one
-// (2M, parity) are consecutive and ordered by W, so in a W-truncated basis the
-// ones that fit the other species' W are the first n of them, and moves
-// between sectors of different W are entries like any other.
+// 4p4n k = 2 against 0.60 ms by the tiled kernel without its pn term.  (At
+// k = 4, 8 the core-grouped kernels take these terms.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -27,74 +25,46 @@
 
 namespace bs {
 
-// The matrix of one species, rows and sources numbered inside the SDs of one (2M, parity).
-void build_like_lists(const Basis &B, int spc, const LikeJumps &L, const LikeCross &X, LikeLists &O)
+// The matrix of one species, sources numbered inside the sector, in order.
+void build_like_lists(const LikeJumps &L, LikeLists &O)
 {
-    const Species &S = B.sp[spc];
     O = LikeLists();
-    // first SD of the (2M, parity) every sector belongs to
-    std::vector<int64_t> first(S.sec.size());
-    for (size_t s = 0; s < S.sec.size(); ++s)
-        first[s] = s > 0 && S.sec[s].twoM == S.sec[s - 1].twoM && S.sec[s].par == S.sec[s - 1].par ? first[s - 1] : S.sec[s].start;
-    std::vector<std::vector<std::pair<int32_t, double>>> cross(X.cls.empty() ? 0 : S.bits.size());
-    for (const LikeCrossClass &c : X.cls) {
-        const Sector &D = S.sec[(size_t)c.s_dst], &Q = S.sec[(size_t)c.s_src];
-        for (int64_t r = 0; r < D.count; ++r)
-            for (int64_t e = X.ptr[(size_t)(c.ptr_off + r)]; e < X.ptr[(size_t)(c.ptr_off + r + 1)]; ++e)
-                cross[(size_t)(D.start + r)].push_back({(int32_t)(Q.start + X.src[(size_t)e] - first[(size_t)c.s_dst]), X.coef[(size_t)e]});
-    }
-    O.ptr.push_back(0);
-    for (size_t g = 0; g < S.bits.size(); ++g) {
-        const size_t s = (size_t)S.sec_of_sd[g];
-        std::vector<std::pair<int32_t, double>> v;
-        for (int64_t e = L.ptr[g]; e < L.ptr[g + 1]; ++e)
-            v.push_back({(int32_t)(S.sec[s].start + L.src[(size_t)e] - first[s]), L.coef[(size_t)e]});
-        if (!cross.empty()) v.insert(v.end(), cross[g].begin(), cross[g].end());
-        std::sort(v.begin(), v.end(), [](const auto &a, const auto &b) { return a.first < b.first; });
-        for (const auto &e : v) O.ent.push_back(LikeEnt{e.first, (float)e.second});
-        O.ptr.push_back((int64_t)O.ent.size());
+    O.ptr = L.ptr;
+    std::vector<std::pair<int32_t, float>> v;
+    for (size_t g = 0; g + 1 < L.ptr.size(); ++g) {
+        v.clear();
+        for (int64_t e = L.ptr[g]; e < L.ptr[g + 1]; ++e) v.push_back({L.src[(size_t)e], (float)L.coef[(size_t)e]});
+        std::sort(v.begin(), v.end());
+        for (const auto &e : v) O.ent.push_back(LikeEnt{e.first, e.second});
     }
 }
 
-// Panels of every (2M, parity) of the acting species and sector of the other: pos SDs of the other each.
-void build_like_panels(const Basis &B, int spc, int pos, LikePanels &O)
+// Panels of every block: pos SDs of the other species each, the widest matrices first.
+void build_like_panels(const Basis &B, int spc, int pos, std::vector<LikePanel> &O, int &max_n)
 {
-    O = LikePanels();
-    const Species &S = B.sp[spc], &Q = B.sp[1 - spc];
-    struct U { double cost; LikePanel p; };
-    std::vector<U> units;
-    for (size_t q = 0; q < Q.sec.size(); ++q) {
-        // the acting species' sectors that pair with q, consecutive in its SD order
+    O.clear();
+    max_n = 0;
+    for (const Block &K : B.blocks) {
         LikePanel p = {};
-        p.piece0 = (int)O.pieces.size();
-        int64_t first = -1;
-        for (size_t s = 0; s < S.sec.size(); ++s) {
-            const int b = spc == 0 ? B.block_of((int)s, (int)q) : B.block_of((int)q, (int)s);
-            if (b < 0) continue;
-            const Block &K = B.blocks[(size_t)b];
-            if (first < 0) first = S.sec[s].start;
-            O.pieces.push_back(LikePiece{(int)(S.sec[s].start - first), (int)S.sec[s].count, K.off, (int)K.nN, 0});
-            p.n = (int)(S.sec[s].start - first + S.sec[s].count);
-        }
-        p.npiece = (int)O.pieces.size() - p.piece0;
-        if (!p.npiece) continue;
-        p.row0 = first;
-        O.max_n = std::max(O.max_n, p.n);
-        for (int64_t c = 0; c < Q.sec[q].count; c += pos) {
+        p.off = K.off;
+        p.nN = (int)K.nN;
+        p.n = (int)(spc == 0 ? K.nP : K.nN);
+        p.row0 = B.sp[spc].sec[(size_t)(spc == 0 ? K.ps : K.ns)].start;
+        max_n = std::max(max_n, p.n);
+        const int64_t other = spc == 0 ? K.nN : K.nP;
+        for (int64_t c = 0; c < other; c += pos) {
             p.pos0 = (int)c;
-            p.npos = (int)std::min<int64_t>(pos, Q.sec[q].count - c);
-            units.push_back(U{(double)p.n, p});
+            p.npos = (int)std::min<int64_t>(pos, other - c);
+            O.push_back(p);
         }
     }
-    std::stable_sort(units.begin(), units.end(), [](const U &a, const U &b) { return a.cost > b.cost; });
-    for (const U &u : units) O.panels.push_back(u.p);
+    std::stable_sort(O.begin(), O.end(), [](const LikePanel &a, const LikePanel &b) { return a.n > b.n; });
 }
 
 namespace {
 
 struct LikeArgs {
     const LikePanel *panels;
-    const LikePiece *pieces;
     const int64_t *ptr;
     const LikeEnt *ent;
     const float *part;     // pp: partial vectors to add, nz of them
@@ -114,105 +84,97 @@ __global__ void __launch_bounds__(1024) hx_like_kernel(LikeArgs A, const float *
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     LikeEnt *buf = reinterpret_cast<LikeEnt *>(sm) + warp * 32;   // this warp's list entries
     float *X = sm + (blockDim.x >> 5) * 64;
-    const LikePiece *pc = A.pieces + P.piece0;
-    for (int i = 0; i < P.npiece; ++i) {
-        const LikePiece Q = pc[i];
-        if constexpr (NN) {
-            // (position r, SDs q): runs of consecutive q
-            const int run = Q.n * K;
-            for (int r = warp; r < P.npos; r += nw) {
-                const float *s = x + (Q.off + (int64_t)(P.pos0 + r) * Q.nN) * K;
-                for (int f = lane; f < run; f += 32) X[(Q.g0 + f / K) * LD + r * K + f % K] = __ldg(s + f);
-            }
-        } else {
-            const int w = P.npos * K;
-            for (int g = warp; g < Q.n; g += nw) {
-                const float *s = x + (Q.off + (int64_t)g * Q.nN + P.pos0) * K;
+    if constexpr (NN) {
+        // (position r, SDs q): runs of consecutive q
+        const int run = P.n * K;
+        for (int r = warp; r < P.npos; r += nw) {
+            const float *s = x + (P.off + (int64_t)(P.pos0 + r) * P.nN) * K;
+            for (int f = lane; f < run; f += 32) X[f / K * LD + r * K + f % K] = __ldg(s + f);
+        }
+    } else {
+        const int w = P.npos * K;
+        for (int g = warp; g < P.n; g += nw) {
+            const float *s = x + (P.off + (int64_t)g * P.nN + P.pos0) * K;
 #pragma unroll
-                for (int v = 0; v < V; ++v)
-                    if (lane + 32 * v < w) X[(Q.g0 + g) * LD + lane + 32 * v] = __ldg(s + lane + 32 * v);
-            }
+            for (int v = 0; v < V; ++v)
+                if (lane + 32 * v < w) X[g * LD + lane + 32 * v] = __ldg(s + lane + 32 * v);
         }
     }
     __syncthreads();
     const float *Xl = X + lane * V;
-    for (int i = 0; i < P.npiece; ++i) {
-        const LikePiece Q = pc[i];
-        int g = warp + nw * (int)blockIdx.y;   // grid.y CTAs share a panel's rows
-        int64_t e0 = 0, e1 = 0;
-        LikeEnt nx{0, 0.0f};              // this lane's entry of the next batch
-        if (g < Q.n) {
-            e0 = A.ptr[P.row0 + Q.g0 + g];
-            e1 = A.ptr[P.row0 + Q.g0 + g + 1];
-            if (e0 + lane < e1) nx = A.ent[e0 + lane];
-        }
-        while (g < Q.n) {
-            float2 acc = make_float2(0.0f, 0.0f);
-            const int gd = g;
-            bool more = true;
-            while (more) {
-                const int cnt = (int)min((int64_t)32, e1 - e0);
-                __syncwarp();
-                buf[lane] = nx;
-                __syncwarp();
-                // the next batch: of this row, or the first of the warp's next row
-                e0 += 32;
-                if (e0 >= e1) {
-                    more = false;
-                    g += nw * (int)gridDim.y;
-                    if (g < Q.n) {
-                        e0 = A.ptr[P.row0 + Q.g0 + g];
-                        e1 = A.ptr[P.row0 + Q.g0 + g + 1];
-                    }
+    int g = warp + nw * (int)blockIdx.y;   // grid.y CTAs share a panel's rows
+    int64_t e0 = 0, e1 = 0;
+    LikeEnt nx{0, 0.0f};              // this lane's entry of the next batch
+    if (g < P.n) {
+        e0 = A.ptr[P.row0 + g];
+        e1 = A.ptr[P.row0 + g + 1];
+        if (e0 + lane < e1) nx = A.ent[e0 + lane];
+    }
+    while (g < P.n) {
+        float2 acc = make_float2(0.0f, 0.0f);
+        const int gd = g;
+        bool more = true;
+        while (more) {
+            const int cnt = (int)min((int64_t)32, e1 - e0);
+            __syncwarp();
+            buf[lane] = nx;
+            __syncwarp();
+            // the next batch: of this row, or the first of the warp's next row
+            e0 += 32;
+            if (e0 >= e1) {
+                more = false;
+                g += nw * (int)gridDim.y;
+                if (g < P.n) {
+                    e0 = A.ptr[P.row0 + g];
+                    e1 = A.ptr[P.row0 + g + 1];
                 }
-                if (g < Q.n && e0 + lane < e1) nx = A.ent[e0 + lane];
-                // entries in pairs: two per broadcast read
-                auto one = [&](int src, float c) {
-                    if (src >= P.n) return;   // a state the truncation leaves out (uniform)
-                    if constexpr (V == 2) {
-                        const float2 v = *reinterpret_cast<const float2 *>(Xl + src * LD);
-                        acc = __ffma2_rn(make_float2(c, c), v, acc);
-                    } else {
-                        acc.x = fmaf(c, Xl[src * LD], acc.x);
-                    }
-                };
-                const int4 *b2 = reinterpret_cast<const int4 *>(buf);
-                int j = 0;
-#pragma unroll 4
-                for (; j + 2 <= cnt; j += 2) {
-                    const int4 q = b2[j >> 1];
-                    one(q.x, __int_as_float(q.y));
-                    one(q.z, __int_as_float(q.w));
-                }
-                if (j < cnt) one(buf[j].src, buf[j].coef);
             }
-            // store: nn writes its rows, pp adds them and the partial vectors
-#pragma unroll
-            for (int v = 0; v < V; v += (K > 1 ? V : 1)) {
-                const int f = lane * V + v, c = f / K;
-                if (c >= P.npos) continue;
-                constexpr bool two = V == 2 && K > 1;
-                if constexpr (NN) {
-                    float *o = y + (Q.off + (int64_t)(P.pos0 + c) * Q.nN + gd) * K + f % K;
-                    if constexpr (two) *reinterpret_cast<float2 *>(o) = acc;
-                    else *o = v ? acc.y : acc.x;
+            if (g < P.n && e0 + lane < e1) nx = A.ent[e0 + lane];
+            // entries in pairs: two per broadcast read
+            auto one = [&](int src, float c) {
+                if constexpr (V == 2) {
+                    const float2 v = *reinterpret_cast<const float2 *>(Xl + src * LD);
+                    acc = __ffma2_rn(make_float2(c, c), v, acc);
                 } else {
-                    const int64_t at = (Q.off + (int64_t)gd * Q.nN + P.pos0) * K + f;
-                    if constexpr (two) {
-                        float2 s = *reinterpret_cast<const float2 *>(y + at);
-                        s.x += acc.x;
-                        s.y += acc.y;
-                        for (int t = 0; t < A.nz; ++t) {
-                            const float2 p = __ldg(reinterpret_cast<const float2 *>(A.part + t * A.pstride + at));
-                            s.x += p.x;
-                            s.y += p.y;
-                        }
-                        *reinterpret_cast<float2 *>(y + at) = s;
-                    } else {
-                        float s = y[at] + (v ? acc.y : acc.x);
-                        for (int t = 0; t < A.nz; ++t) s += __ldg(A.part + t * A.pstride + at);
-                        y[at] = s;
+                    acc.x = fmaf(c, Xl[src * LD], acc.x);
+                }
+            };
+            const int4 *b2 = reinterpret_cast<const int4 *>(buf);
+            int j = 0;
+#pragma unroll 4
+            for (; j + 2 <= cnt; j += 2) {
+                const int4 q = b2[j >> 1];
+                one(q.x, __int_as_float(q.y));
+                one(q.z, __int_as_float(q.w));
+            }
+            if (j < cnt) one(buf[j].src, buf[j].coef);
+        }
+        // store: nn writes its rows, pp adds them and the partial vectors
+#pragma unroll
+        for (int v = 0; v < V; v += (K > 1 ? V : 1)) {
+            const int f = lane * V + v, c = f / K;
+            if (c >= P.npos) continue;
+            constexpr bool two = V == 2 && K > 1;
+            if constexpr (NN) {
+                float *o = y + (P.off + (int64_t)(P.pos0 + c) * P.nN + gd) * K + f % K;
+                if constexpr (two) *reinterpret_cast<float2 *>(o) = acc;
+                else *o = v ? acc.y : acc.x;
+            } else {
+                const int64_t at = (P.off + (int64_t)gd * P.nN + P.pos0) * K + f;
+                if constexpr (two) {
+                    float2 s = *reinterpret_cast<const float2 *>(y + at);
+                    s.x += acc.x;
+                    s.y += acc.y;
+                    for (int t = 0; t < A.nz; ++t) {
+                        const float2 p = __ldg(reinterpret_cast<const float2 *>(A.part + t * A.pstride + at));
+                        s.x += p.x;
+                        s.y += p.y;
                     }
+                    *reinterpret_cast<float2 *>(y + at) = s;
+                } else {
+                    float s = y[at] + (v ? acc.y : acc.x);
+                    for (int t = 0; t < A.nz; ++t) s += __ldg(A.part + t * A.pstride + at);
+                    y[at] = s;
                 }
             }
         }
@@ -233,14 +195,13 @@ template <int K, int PW, bool NN>
 cudaError_t launch_like_t(int dev, const Device::LikeDev &L, const float *x, float *y, const float *part, int nz, int64_t pstride,
                           cudaStream_t s)
 {
-    constexpr int slot = (PW == 64 ? 0 : 4) + (K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : 3);
     const int th = like_threads(L.max_n);
     const size_t smem = like_smem(L.max_n, PW, th);
     auto kern = hx_like_kernel<K, PW, NN>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    LikeArgs A{L.panels[slot & 3], L.pieces, L.ptr, L.ent, part, nz, pstride, L.max_n};
-    const int np = L.npanels[slot & 3];
+    LikeArgs A{L.panels[K - 1], L.ptr, L.ent, part, nz, pstride, L.max_n};
+    const int np = L.npanels[K - 1];
     if (np <= 0) return cudaSuccess;
     // several CTAs to a panel, each with some of its rows, until there are four for every
     // place on the chip (a panel is loaded in a fortieth of the time its rows take) or a
@@ -279,12 +240,7 @@ bool like_applies(const bs_ctx *c) { return c->dev.like[0].pw > 0 && c->dev.like
 cudaError_t launch_hx_like(const bs_ctx *c, const float *x, float *y, int k, cudaStream_t s, const float *part, int nz)
 {
     const int64_t ps = c->basis.dim * k;
-    switch (k) {
-    case 1: return launch_like_k<1>(c->dev, x, y, part, nz, ps, s);
-    case 2: return launch_like_k<2>(c->dev, x, y, part, nz, ps, s);
-    case 4: return launch_like_k<4>(c->dev, x, y, part, nz, ps, s);
-    default: return launch_like_k<8>(c->dev, x, y, part, nz, ps, s);
-    }
+    return k == 1 ? launch_like_k<1>(c->dev, x, y, part, nz, ps, s) : launch_like_k<2>(c->dev, x, y, part, nz, ps, s);
 }
 
 }  // namespace bs

@@ -1,5 +1,5 @@
 // pn term of y = H x by pairs of cores (sm_103a): for one proton core cp and
-// one group of neutron cores cn of equal (2M, parity, W),
+// one group of neutron cores cn of equal (2M, parity),
 //   G[ij][cn] = sum_kl W[ij][kl] X[kl][cn],  X[kl][cn] = sign x[cp+k, cn+l],
 // a dense matrix product with one W for all of them (bs_pair.cpp), whose
 // result is added to the rows cp + i of y at column cn + j.  Against the
@@ -24,7 +24,7 @@
 // added to the group's own rows of Y, so groups never touch the same element
 // and one group's adds run under the others' multiply-adds.  Inside a group
 // the adds go in rounds: rows whose neutron state j has the same place among
-// the states of its (2m, parity, w) meet a column once, so no two threads add
+// the states of its (2m, parity) meet a column once, so no two threads add
 // to one element in a round.  No atomics, a fixed order of additions.  Waits
 // are bounded: on expiry the CTA records BS_ETIMEOUT, stops waiting and runs
 // to its end (its rows are then garbage, as the status says).

@@ -273,18 +273,12 @@ struct PairItems {
 };
 
 // Like-particle matrices with uniform lists (bs_hx_like.cu).
-struct LikeEnt { int32_t src; float coef; };     // source SD among those of its (2M, parity)
+struct LikeEnt { int32_t src; float coef; };     // source SD in its sector
 struct LikeLists {
     std::vector<int64_t> ptr;                    // per SD of the species
     std::vector<LikeEnt> ent;
 };
-struct LikePiece { int g0, n; int64_t off; int nN, pad; };   // SDs g0 .. g0 + n - 1 of the panel: one block
-struct LikePanel { int64_t row0; int n, pos0, npos, piece0, npiece, pad; };
-struct LikePanels {
-    std::vector<LikePanel> panels;
-    std::vector<LikePiece> pieces;
-    int max_n = 0;
-};
+struct LikePanel { int64_t off, row0; int nN, n, pos0, npos; };   // a block's n SDs by npos of the other species'; row0: the first of the n
 
 struct Tables {
     PairTables pair;
@@ -453,13 +447,12 @@ struct Device {
     // neutron like-particle kernel over tiles of R proton rows (R = 2, 4): (block, first row)
     int2 *nntasks2 = nullptr, *nntasks4 = nullptr;
     int nnntasks2 = 0, nnntasks4 = 0;
-    // like-particle matrices: protons, neutrons; panels for k = 1, 2, 4, 8
+    // like-particle matrices: protons, neutrons; panels for k = 1, 2
     struct LikeDev {
         int64_t *ptr = nullptr;
         LikeEnt *ent = nullptr;
-        LikePiece *pieces = nullptr;
-        LikePanel *panels[4] = {nullptr, nullptr, nullptr, nullptr};
-        int npanels[4] = {0, 0, 0, 0}, max_n = 0, pw = 0;
+        LikePanel *panels[2] = {nullptr, nullptr};
+        int npanels[2] = {0, 0}, max_n = 0, pw = 0;
     } like[2];
     // pair-core pn kernel: items for 4, 2 and 1 components at a time (shared where the rows of a proton core fit)
     struct PairDev {
@@ -524,8 +517,8 @@ void build_interaction_derivatives(const Basis &B, const Interaction &I, const s
                                    std::vector<WTerm> &pn);
 void release_adj(AdjPlan &P);
 int build_tables(const Basis &B, const Interaction &I, Tables &T, std::string &err, int grid = 152);
-void build_like_lists(const Basis &B, int spc, const LikeJumps &L, const LikeCross &X, LikeLists &O);
-void build_like_panels(const Basis &B, int spc, int pos, LikePanels &O);
+void build_like_lists(const LikeJumps &L, LikeLists &O);
+void build_like_panels(const Basis &B, int spc, int pos, std::vector<LikePanel> &O, int &max_n);
 int like_panel_width(int max_n);
 bool like_applies(const bs_ctx *ctx);
 void build_pair_tables(const Basis &B, const Interaction &I, PairTables &T, int64_t max_cols);

@@ -1,14 +1,14 @@
 """Host tables of the pair-core pn kernel (bs_pair.cpp), checked on the CPU:
 walking them as the kernel does, with the like-particle terms from the
 destination lists, gives the same H x as the general tables (which
-test_host_tables.py and test_truncation.py pin to the oracle), plain and
-W-truncated, and every index stays inside its buffer."""
+test_host_tables.py pins to the oracle), and every index stays inside its
+buffer."""
 import numpy as np
 import pytest
 
 from paper_1801_08432_gb300 import _native as N
 from paper_1801_08432_gb300 import inputs as I
-from tests.test_truncation import truncated_tables_matvec
+from tests.test_host_tables import tables_matvec
 
 REC = np.dtype([("xoff", np.uint32), ("yoff", np.uint32), ("srec", np.uint32), ("wj", np.uint32)])
 ROW = np.dtype([("elem", np.int64), ("ycol", np.int32), ("n", np.int32), ("part", np.int32), ("state", np.int32),
@@ -81,31 +81,27 @@ def pair_matvec(c, x, Z, cp):
     return part.sum(axis=0)
 
 
-SPACES = [("sd", 2, 2, 0, None), ("sd", 3, 2, 1, None), ("sd", 1, 1, 0, None), ("sd", 5, 1, 2, None), ("p", 3, 3, 0, None),
-          ("pf", 2, 2, 2, None), ("sd", 3, 3, 0, 2), ("pf", 2, 1, 1, 1), ("pf", 2, 2, 0, 2)]
+SPACES = [("sd", 2, 2, 0), ("sd", 3, 2, 1), ("sd", 1, 1, 0), ("sd", 5, 1, 2), ("p", 3, 3, 0),
+          ("pf", 2, 2, 2), ("pf", 2, 1, 1)]
 
 
-@pytest.mark.parametrize("name,Z,Nn,twoM,excite", SPACES)
+@pytest.mark.parametrize("name,Z,Nn,twoM", SPACES)
 @pytest.mark.parametrize("cp", [1, 4])
-def test_pair_tables_reproduce_the_pn_term(name, Z, Nn, twoM, excite, cp):
+def test_pair_tables_reproduce_the_pn_term(name, Z, Nn, twoM, cp):
     orbits, spe, tb = I.space(name)
     par = (-1) ** (((Z + Nn) * (orbits[0].l % 2)) % 2)
-    orbits = [I.Orbit(o.n, o.l, o.twoj, 0 if a == 0 else 1) for a, o in enumerate(orbits)]
-    c = N.make(orbits, spe, tb, Z, Nn, twoM, par, device=-1, max_excite=excite)
+    c = N.make(orbits, spe, tb, Z, Nn, twoM, par, device=-1)
     x = I.random_block(c.dim, 1, seed=5)[:, 0]
     y = pair_matvec(c, x, Z, cp) + like_matvec(c, x)
-    ref = truncated_tables_matvec(c, x)
+    ref = tables_matvec(c, x)
     assert np.max(np.abs(y - ref)) <= 1e-12 * np.max(np.abs(ref))
 
 
 def like_matvec(c, x):
-    """The pp and nn terms of y = H x from the destination lists, other sectors' moves included."""
+    """The pp and nn terms of y = H x from the destination lists."""
     B = c.export_basis()
     pp, pps, ppc = c.table("pp_ptr", np.int64), c.table("pp_src", np.int32), c.table("pp_coef", np.float64)
     nn, nns, nnc = c.table("nn_ptr", np.int64), c.table("nn_src", np.int32), c.table("nn_coef", np.float64)
-    links = c.table("llinks", np.int64).reshape(-1, 4)
-    xt = {0: [c.table("ppx_" + q, t) for q, t in (("ptr", np.int64), ("src", np.int32), ("coef", np.float64))],
-          1: [c.table("nnx_" + q, t) for q, t in (("ptr", np.int64), ("src", np.int32), ("coef", np.float64))]}
     y = np.zeros_like(x)
     V = lambda a, b: a[int(B["blocks"][b][2]):][:shape(b)[0] * shape(b)[1]].reshape(shape(b))
     shape = lambda b: (int(B["p_sec"][B["blocks"][b][0]][3]), int(B["n_sec"][B["blocks"][b][1]][3]))
@@ -118,13 +114,4 @@ def like_matvec(c, x):
         for q in range(X.shape[1]):
             e = slice(nn[n0 + q], nn[n0 + q + 1])
             Y[:, q] += X[:, nns[e]] @ nnc[e]
-    for d, s, spc, po in links:
-        X, Y = V(x, s), V(y, d)
-        ptr, src, cf = xt[int(spc)]
-        for r in range(Y.shape[int(spc)]):
-            e = slice(ptr[po + r], ptr[po + r + 1])
-            if spc == 0:
-                Y[r] += cf[e] @ X[src[e]]
-            else:
-                Y[:, r] += X[:, src[e]] @ cf[e]
     return y
