@@ -278,7 +278,7 @@ int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std
     if ((rc = put(D, D.pps_w32, f.data(), f.size(), err))) return rc;
     f = cast<float>(T.pdiag);
     if ((rc = put(D, D.pdiag32, f.data(), f.size(), err))) return rc;
-    for (int R : {2, 4}) {
+    for (int R : {2, 3, 4}) {
         // row tiles of the neutron like-particle kernel, widest sectors first
         std::vector<int2> nt;
         std::vector<size_t> ord(B.blocks.size());
@@ -286,8 +286,8 @@ int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std
         std::stable_sort(ord.begin(), ord.end(), [&](size_t a, size_t b2) { return B.blocks[a].nN > B.blocks[b2].nN; });
         for (size_t b2 : ord)
             for (int64_t r = 0; r < B.blocks[b2].nP; r += R) nt.push_back(make_int2((int)b2, (int)r));
-        int2 *&dst = R == 2 ? D.nntasks2 : D.nntasks4;
-        (R == 2 ? D.nnntasks2 : D.nnntasks4) = (int)nt.size();
+        int2 *&dst = R == 2 ? D.nntasks2 : R == 3 ? D.nntasks3 : D.nntasks4;
+        (R == 2 ? D.nnntasks2 : R == 3 ? D.nnntasks3 : D.nnntasks4) = (int)nt.size();
         if ((rc = put(D, dst, nt.data(), nt.size(), err))) return rc;
     }
     for (int spc = 0; spc < 2 && T.pair.on; ++spc) {   // like-particle panels

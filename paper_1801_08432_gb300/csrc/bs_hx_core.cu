@@ -454,11 +454,15 @@ struct PPArgs {
 };
 
 // pp term by (Z-2)-proton cores.  The same ring as above; a slot holds one
-// source row and its kPPG signed weights (CTA-uniform: read as broadcasts).
+// source row (of wider sectors the columns of the CTA's current tile) and its
+// kPPG signed weights (CTA-uniform: read as broadcasts).
 // Each thread owns one destination column in natural order (a quarter warp
 // reads eight consecutive 32-byte elements: conflict-free with the lane
 // rotation (lane >> 2) & 1) and applies the element to kPPG destination rows.
-template <int K, int NW, int MINB>
+// With CPT = 2 it owns two, NW * 32 apart, which halves the weights' reads and
+// the slot hand-overs per element.  pf 6p6n k = 4 (3,952 columns): whole rows
+// in each of seven passes 29.6 ms, a tile's columns 17.0, CPT = 2 13.3.
+template <int K, int NW, int MINB, int CPT>
 __global__ void __launch_bounds__((NW + 1) * 32, MINB)
     hx_ppcore_kernel(PPArgs A, const float *__restrict__ x, float *__restrict__ part)
 {
@@ -467,7 +471,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB)
     uint64_t *bars = reinterpret_cast<uint64_t *>(slots + (size_t)A.S * A.slot_elems);
     int *uidp = reinterpret_cast<int *>(bars + 2 * A.S);   // per slot: the unit after the current one
     const uint32_t full0 = su32(bars), empty0 = su32(bars + A.S);
-    constexpr int C = NW * 32;
+    constexpr int C = NW * 32 * CPT;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -524,9 +528,9 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB)
                 rg.next(A.S);
             }
             const int ntile = (nN + C - 1) / C;
-            const uint32_t bytes = (uint32_t)(nN * K * (int)sizeof(float));
             const uint32_t wbytes = (uint32_t)(kPPG * sizeof(float));
-            for (int tile = 0; tile < ntile; ++tile)
+            for (int tile = 0; tile < ntile; ++tile) {
+                const uint32_t bytes = (uint32_t)(min(C, nN - tile * C) * K * (int)sizeof(float));
                 for (int q0 = 0; q0 < nsrc; q0 += 32) {
                     const int32_t myrow = q0 + lane < nsrc ? A.srow[src0 + q0 + lane] : 0;
                     const int cnt = min(32, nsrc - q0);
@@ -544,7 +548,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB)
                                 if (tile == 0 && q0 + j == 0) uidp[s] = un;   // published by the arrive below
                                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                                 bar_expect_tx(fb, bytes + wbytes);
-                                bulk_copy(su32(dst), x + (doff + (int64_t)row * nN) * K, bytes, fb);
+                                bulk_copy(su32(dst), x + (doff + (int64_t)row * nN + tile * C) * K, bytes, fb);
                                 bulk_copy(su32(dst + A.row_stride), A.w + (src0 + q0 + j) * kPPG, wbytes, fb);
                             }
                         }
@@ -557,6 +561,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB)
                         }
                     }
                 }
+            }
         }
         return;
     }
@@ -584,14 +589,15 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB)
         const int64_t doff = ho;
         const int ntile = (nN + C - 1) / C;
         for (int tile = 0; tile < ntile; ++tile) {
-            const int col = tile * C + warp * 32 + lane;
-            const bool active = tile * C + warp * 32 < nN;
-            const int cl = col < nN ? col : nN - 1;
-            float2 acc[kPPG][K / 2];   // packed: components 2j, 2j+1 (in the lane's rotated order)
+            const int tc = min(C, nN - tile * C);   // columns of the tile
+            const bool active = warp * 32 < tc;
+            float2 acc[CPT][kPPG][K / 2];   // packed: components 2j, 2j+1 (in the lane's rotated order)
 #pragma unroll
-            for (int p = 0; p < kPPG; ++p)
+            for (int h = 0; h < CPT; ++h)
 #pragma unroll
-                for (int q = 0; q < K / 2; ++q) acc[p][q] = make_float2(0.0f, 0.0f);
+                for (int p = 0; p < kPPG; ++p)
+#pragma unroll
+                    for (int q = 0; q < K / 2; ++q) acc[h][p][q] = make_float2(0.0f, 0.0f);
             // a unit without sources still takes one (empty) slot: the one with the next unit
             for (int q = 0; q < nsrc || (nsrc == 0 && tile == 0 && q == 0); ++q, rg.next(A.S)) {
                 const int s = rg.s;
@@ -615,14 +621,17 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB)
                         const float4 w4 = *reinterpret_cast<const float4 *>(Xs + A.row_stride + p);
                         w[p] = w4.x; w[p + 1] = w4.y; w[p + 2] = w4.z; w[p + 3] = w4.w;
                     }
-                    float xv[K];
-                    pld<float, K>(Xs, cl, rot, xv);
+                    float xv[CPT][K];
+#pragma unroll
+                    for (int h = 0; h < CPT; ++h) pld<float, K>(Xs, min((h * NW + warp) * 32 + lane, tc - 1), rot, xv[h]);
 #pragma unroll
                     for (int p = 0; p < kPPG; ++p) {
                         const float2 wp = make_float2(w[p], w[p]);
 #pragma unroll
-                        for (int qq = 0; qq < K / 2; ++qq)
-                            acc[p][qq] = __ffma2_rn(wp, make_float2(xv[2 * qq], xv[2 * qq + 1]), acc[p][qq]);
+                        for (int h = 0; h < CPT; ++h)
+#pragma unroll
+                            for (int qq = 0; qq < K / 2; ++qq)
+                                acc[h][p][qq] = __ffma2_rn(wp, make_float2(xv[h][2 * qq], xv[h][2 * qq + 1]), acc[h][p][qq]);
                     }
                 }
                 __syncwarp();
@@ -632,17 +641,20 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB)
 #pragma unroll
             for (int p = 0; p < kPPG; ++p) {
                 const int pk = __shfl_sync(0xffffffffu, rec, p);
-                if (col < nN) {
-                    if (pk < 0) continue;
-                    const int drow = pk >> 8, prt = pk & 255;
+                if (pk < 0) continue;
+                const int drow = pk >> 8, prt = pk & 255;
+#pragma unroll
+                for (int h = 0; h < CPT; ++h) {
+                    const int col = (h * NW + warp) * 32 + lane;
+                    if (col >= tc) continue;
                     float o[K];
 #pragma unroll
                     for (int qq = 0; qq < K / 2; ++qq) {
-                        o[2 * qq] = acc[p][qq].x;
-                        o[2 * qq + 1] = acc[p][qq].y;
+                        o[2 * qq] = acc[h][p][qq].x;
+                        o[2 * qq + 1] = acc[h][p][qq].y;
                     }
                     prot_fix<float, K>(o, rot);
-                    pst<float, K>(part + (int64_t)prt * A.part_stride + (doff + (int64_t)drow * nN + col) * K, o);
+                    pst<float, K>(part + (int64_t)prt * A.part_stride + (doff + (int64_t)drow * nN + tile * C + col) * K, o);
                 }
             }
         }
@@ -906,9 +918,9 @@ cudaError_t launch_nn_t(const bs_ctx *ctx, const float *x, float *out, cudaStrea
     auto kern = hx_nn_rows_kernel<K, R, NW, MINB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    NNArgs A{stage, R == 2 ? Dv.nntasks2 : Dv.nntasks4, Dv.blocks, Dv.pe_perm, Dv.pe_nn_src, Dv.pe_nn_coef32,
+    NNArgs A{stage, R == 2 ? Dv.nntasks2 : R == 3 ? Dv.nntasks3 : Dv.nntasks4, Dv.blocks, Dv.pe_perm, Dv.pe_nn_src, Dv.pe_nn_coef32,
              Dv.pe_nn_sinfo, Dv.pdiag32, Dv.err, row_stride, part, part ? nz : 0, ctx->basis.dim * K};
-    kern<<<R == 2 ? Dv.nnntasks2 : Dv.nnntasks4, NW * 32, smem, s>>>(A, x, out);
+    kern<<<R == 2 ? Dv.nnntasks2 : R == 3 ? Dv.nnntasks3 : Dv.nnntasks4, NW * 32, smem, s>>>(A, x, out);
     return cudaGetLastError();
 }
 
@@ -917,6 +929,7 @@ cudaError_t launch_nn_k(const bs_ctx *ctx, const float *x, float *out, cudaStrea
                        const float *part = nullptr, int nz = 0)
 {
     return R == 2 ? launch_nn_t<K, 2, 2>(ctx, x, out, s, used, part, nz)
+         : R == 3 ? launch_nn_t<K, 3, 1>(ctx, x, out, s, used, part, nz)
                   : launch_nn_t<K, 4, 1>(ctx, x, out, s, used, part, nz);
 }
 
@@ -959,18 +972,18 @@ cudaError_t launch_core_t(const bs_ctx *ctx, const float *x, float *part, cudaSt
     return cudaGetLastError();
 }
 
-template <int K, int NW, int MINB>
+template <int K, int NW, int MINB, int CPT>
 cudaError_t launch_pp_t(const bs_ctx *ctx, const float *x, float *part, cudaStream_t s, size_t target, bool &used)
 {
     const Device &Dv = ctx->dev;
-    const int row_stride = ((Dv.max_nN * K + 31) / 32) * 32;
-    const int slot_elems = row_stride + 32;   // row, kPPG weights, padded to 128 bytes
+    const int row_stride = ((std::min(Dv.max_nN, NW * 32 * CPT) * K + 31) / 32) * 32;
+    const int slot_elems = row_stride + 32;   // a tile's columns of a row, kPPG weights, padded to 128 bytes
     const size_t slot_bytes = (size_t)slot_elems * sizeof(float) + 16;
     const int S = target > 64 ? (int)std::min<size_t>(8, (target - 64) / slot_bytes) : 0;
     used = S >= 2;
     if (!used) return cudaSuccess;
     const size_t smem = (size_t)S * slot_elems * sizeof(float) + 16 * (size_t)S + 64;   // + the slots' next-unit words
-    auto kern = hx_ppcore_kernel<K, NW, MINB>;
+    auto kern = hx_ppcore_kernel<K, NW, MINB, CPT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int nsm = 0, per = 0;
@@ -1070,12 +1083,20 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
     const bool pp = kCoreVariants[v].pp;
     const int R = kCoreVariants[v].nn_rows;
     bool fits = false;
+    int nrow = 0;
     cudaError_t e = cudaSuccess;
     int pv = 0;   // pipelined variant for the like-particle terms: the first that fits
     if (R) {
         e = k == 8 ? launch_nn_k<8>(c, nullptr, nullptr, s, R, fits) : launch_nn_k<4>(c, nullptr, nullptr, s, R, fits);
     } else {
-        for (; pv < pipe_variants() && e == cudaSuccess; ++pv) {
+        // nn by tiles of three or two rows into one more partial vector where they fit (a list entry is read once for
+        // all of them: pf 6p6n k = 4, 17 ms by the row at a time, 14.4 by two, 13.1 by three), else by the first
+        // pipelined variant that fits
+        for (int r = 3; pp && !nrow && r >= 2 && e == cudaSuccess; --r) {
+            e = k == 8 ? launch_nn_k<8>(c, nullptr, nullptr, s, r, fits) : launch_nn_k<4>(c, nullptr, nullptr, s, r, fits);
+            if (fits) nrow = r;
+        }
+        for (; !fits && pv < pipe_variants() && e == cudaSuccess; ++pv) {
             e = launch_hx_pipe_combine(c, nullptr, nullptr, k, dt, s, pv, nullptr, 0, pp, fits);
             if (fits) break;
         }
@@ -1094,8 +1115,10 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
     int nz = c->dev.nz;
     if (pp) {
         if (c->dev.nppunits > 0) {
-            e = k == 8 ? launch_pp_t<8, 18, 1>(c, xf, part, s, kCoreVariants[v].target, used)
-                       : launch_pp_t<4, 18, 1>(c, xf, part, s, kCoreVariants[v].target, used);
+            const size_t tg = kCoreVariants[v].target;
+            e = k == 8 ? launch_pp_t<8, 18, 1, 1>(c, xf, part, s, tg, used)
+              : c->dev.max_nN > 18 * 32 ? launch_pp_t<4, 18, 1, 2>(c, xf, part, s, tg, used)
+                                        : launch_pp_t<4, 18, 1, 1>(c, xf, part, s, tg, used);
             if (e != cudaSuccess) return e;
             if (!used) return cudaErrorInvalidConfiguration;   // the pn kernel with the same budget fitted
         }
@@ -1110,7 +1133,12 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
         if (e != cudaSuccess) return e;
         return used ? cudaGetLastError() : cudaSuccess;
     }
-    e = launch_hx_pipe_combine(c, x, y, k, dt, s, pv, part, -1 - nz, pp, used);
+    if (nrow) {
+        float *out = part + (int64_t)nz * c->basis.dim * k;
+        e = k == 8 ? launch_nn_k<8>(c, xf, out, s, nrow, used) : launch_nn_k<4>(c, xf, out, s, nrow, used);
+    } else {
+        e = launch_hx_pipe_combine(c, x, y, k, dt, s, pv, part, -1 - nz, pp, used);
+    }
     if (e != cudaSuccess || !used) return e;
     const int64_t n4 = c->basis.dim * k / 4;
     int nsm = 0;

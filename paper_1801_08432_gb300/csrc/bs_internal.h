@@ -444,9 +444,9 @@ struct Device {
     int32_t *pps_row = nullptr;
     float *pps_w32 = nullptr, *pdiag32 = nullptr;
     int nppunits = 0, nzpp = 0;
-    // neutron like-particle kernel over tiles of R proton rows (R = 2, 4): (block, first row)
-    int2 *nntasks2 = nullptr, *nntasks4 = nullptr;
-    int nnntasks2 = 0, nnntasks4 = 0;
+    // neutron like-particle kernel over tiles of R proton rows (R = 2, 3, 4): (block, first row)
+    int2 *nntasks2 = nullptr, *nntasks3 = nullptr, *nntasks4 = nullptr;
+    int nnntasks2 = 0, nnntasks3 = 0, nnntasks4 = 0;
     // like-particle matrices: protons, neutrons; panels for k = 1, 2
     struct LikeDev {
         int64_t *ptr = nullptr;
