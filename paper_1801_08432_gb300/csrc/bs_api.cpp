@@ -80,11 +80,12 @@ static void make_tasks(const Basis &B, const Tables &T, int tile, std::vector<De
 {
     struct C { double cost; DevTask t; };
     std::vector<C> v;
+    int list = 0;
     for (size_t b = 0; b < B.blocks.size(); ++b) {
         const Block &D = B.blocks[b];
         const Sector &PS = B.sp[0].sec[D.ps], &NS = B.sp[1].sec[D.ns];
         double nn_avg = (double)(T.nn.ptr[NS.start + NS.count] - T.nn.ptr[NS.start]) / (double)std::max<int64_t>(1, NS.count);
-        for (int64_t r = 0; r < D.nP; ++r) {
+        for (int64_t r = 0; r < D.nP; ++r, ++list) {
             double per_col = (double)(T.pp.ptr[PS.start + r + 1] - T.pp.ptr[PS.start + r]) + nn_avg;
             for (int64_t L = T.links_of_block[b]; L < T.links_of_block[b + 1]; ++L) {
                 const PnLink &lk = T.links[(size_t)L];
@@ -95,13 +96,47 @@ static void make_tasks(const Basis &B, const Tables &T, int tile, std::vector<De
             }
             for (int64_t c0 = 0; c0 < D.nN; c0 += tile) {
                 int64_t cols = std::min<int64_t>(tile, D.nN - c0);
-                v.push_back(C{per_col * (double)cols, DevTask{(int)b, (int)r, (int)c0, 0}});
+                v.push_back(C{per_col * (double)cols, DevTask{(int)b, (int)r, (int)c0, list}});
             }
         }
     }
     std::stable_sort(v.begin(), v.end(), [](const C &a, const C &b) { return a.cost > b.cost; });
     tasks.resize(v.size());
     for (size_t i = 0; i < v.size(); ++i) tasks[i] = v[i].t;
+}
+
+// The proton one-body jumps into every (block, row) from all linked blocks, in the order of the links.
+static void make_row_jumps(const Basis &B, const Tables &T, std::vector<int64_t> &ptr, std::vector<RowJump> &jumps)
+{
+    ptr.assign(1, 0);
+    for (size_t b = 0; b < B.blocks.size(); ++b)
+        for (int64_t r = 0; r < B.blocks[b].nP; ++r) {
+            int64_t n = 0;
+            for (int64_t L = T.links_of_block[b]; L < T.links_of_block[b + 1]; ++L) {
+                const int64_t *p = T.p1.ptr.data() + T.p1.cls[(size_t)T.links[(size_t)L].pcls].ptr_off + r;
+                n += p[1] - p[0];
+            }
+            ptr.push_back(ptr.back() + n);
+        }
+    jumps.resize((size_t)ptr.back());
+    size_t row0 = 0;
+    for (size_t b = 0; b < B.blocks.size(); row0 += (size_t)B.blocks[b].nP, ++b) {
+        const int64_t nP = B.blocks[b].nP;
+#pragma omp parallel for schedule(static)
+        for (int64_t r = 0; r < nP; ++r) {
+            RowJump *o = jumps.data() + ptr[row0 + (size_t)r];
+            for (int64_t L = T.links_of_block[b]; L < T.links_of_block[b + 1]; ++L) {
+                const PnLink &lk = T.links[(size_t)L];
+                const Block &S = B.blocks[(size_t)lk.src_block];
+                const int64_t *p = T.p1.ptr.data() + T.p1.cls[(size_t)lk.pcls].ptr_off + r;
+                for (int64_t u = p[0]; u < p[1]; ++u) {
+                    const uint32_t e = T.p1.ent[(size_t)u];
+                    *o++ = RowJump{S.off + (int64_t)(e & 0xFFFFu) * S.nN, (uint32_t)T.n1.cls[(size_t)lk.ncls].ptr_off,
+                                   (uint32_t)(lk.w_off + (int64_t)((e >> 16) & 0x7FFFu) * lk.nb) | (e & 0x80000000u)};
+                }
+            }
+        }
+    }
 }
 
 // One CTA per destination proton row for the row kernel, largest work first.
@@ -181,6 +216,13 @@ int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std
     if ((rc = put(D, D.blocks, blocks.data(), blocks.size(), err))) return rc;
     if ((rc = put(D, D.links, links.data(), links.size(), err))) return rc;
     if ((rc = put(D, D.tasks, tasks.data(), tasks.size(), err))) return rc;
+    {
+        std::vector<int64_t> jp;
+        std::vector<RowJump> jumps;
+        make_row_jumps(B, T, jp, jumps);
+        if ((rc = put(D, D.jump_ptr, jp.data(), jp.size(), err))) return rc;
+        if ((rc = put(D, D.jumps, jumps.data(), jumps.size(), err))) return rc;
+    }
     if ((rc = put(D, D.pp_ptr, T.pp.ptr.data(), T.pp.ptr.size(), err))) return rc;
     if ((rc = put(D, D.pp_src, T.pp.src.data(), T.pp.src.size(), err))) return rc;
     if ((rc = put(D, D.nn_ptr, T.nn.ptr.data(), T.nn.ptr.size(), err))) return rc;

@@ -78,17 +78,18 @@ __device__ __forceinline__ void stk(T *__restrict__ p, const T (&r)[K])
 struct HxArgs {
     const DevTask *tasks;
     const DevBlock *blocks;
-    const DevLink *links;
-    const int64_t *pp_ptr, *nn_ptr, *p1_ptr, *n1_ptr;
+    const int64_t *pp_ptr, *nn_ptr, *n1_ptr;
     const int32_t *pp_src, *nn_src;
-    const uint32_t *p1_ent, *n1_ent;
+    const uint32_t *n1_ent;
+    const RowJump *jumps;
+    const int64_t *jump_ptr;
     const DevLLink *llinks;
     const int64_t *ppx_ptr, *nnx_ptr;
     const int32_t *ppx_src, *nnx_src;
 };
 
 // A CTA's warps beyond the tile's columns form further groups (G in all): group
-// g takes every G-th like-particle entry and every G-th pn link, and the
+// g takes every G-th like-particle entry and proton jump, and the
 // groups' sums meet in shared memory, in the order of the groups.  A thread's
 // chain of dependent loads (list pointer, entry, element) is what bounds the
 // kernel on small bases and narrow sectors, where the extra warps cost
@@ -165,37 +166,45 @@ __global__ void __launch_bounds__(NT) hx_fused_kernel(HxArgs A, const T *__restr
                 }
             }
         }
-        // pn: proton one-body jump x neutron one-body jump, per linked source block
-        for (int L = D.link_begin + g; L < D.link_end; L += G) {
-            const DevLink lk = A.links[L];
-            const int64_t pb = A.p1_ptr[lk.p_ptr_off + t.row], pe = A.p1_ptr[lk.p_ptr_off + t.row + 1];
-            const int64_t nb0 = A.n1_ptr[lk.n_ptr_off + col], ne0 = A.n1_ptr[lk.n_ptr_off + col + 1];
-            if (pb == pe || nb0 == ne0) continue;
-            const DevBlock S = A.blocks[lk.src_block];
-            const T *W = wpn + lk.w_off;
-            for (int64_t u = pb; u < pe; ++u) {
-                const uint32_t ep = A.p1_ent[u];
-                const T *xr = x + (S.off + (int64_t)(ep & 0xFFFFu) * S.nN) * K;
-                const T *Wa = W + (int64_t)((ep >> 16) & 0x7FFFu) * lk.nb;
-                T part[K];
+        // pn: the row's proton one-body jumps from every linked block, in one list, each times the column's neutron
+        // one-body jumps of that link.  The next jump's record and list bounds are on the way while this one runs: link by
+        // link, with its block and two pointers to read before any jump, sd 4p4n k = 4 took 34 us (27 now), pf 5p4n
+        // 4p-4h (269 blocks) 2.53 ms (2.07).
+        int64_t j = A.jump_ptr[t.list] + g;
+        const int64_t j1 = A.jump_ptr[t.list + 1];
+        RowJump nj{};
+        int64_t nb0 = 0, ne0 = 0;
+        auto fetch = [&]() {
+            nj = A.jumps[j];
+            nb0 = A.n1_ptr[nj.nptr + col];
+            ne0 = A.n1_ptr[nj.nptr + col + 1];
+        };
+        if (j < j1) fetch();
+        while (j < j1) {
+            const RowJump J = nj;
+            const int64_t v0 = nb0, v1 = ne0;
+            j += G;
+            if (j < j1) fetch();
+            const T *xr = x + J.xoff * K;
+            const T *Wa = wpn + (J.w & 0x7FFFFFFFu);
+            T part[K];
 #pragma unroll
-                for (int q = 0; q < K; ++q) part[q] = T(0);
+            for (int q = 0; q < K; ++q) part[q] = T(0);
 #pragma unroll 2
-                for (int64_t v = nb0; v < ne0; ++v) {
-                    const uint32_t en = A.n1_ent[v];
-                    T w = __ldg(Wa + ((en >> 16) & 0x7FFFu));
-                    if (en >> 31) w = -w;
-                    ldk<T, K>(xr + (int64_t)(en & 0xFFFFu) * K, xv);
+            for (int64_t v = v0; v < v1; ++v) {
+                const uint32_t en = A.n1_ent[v];
+                T w = __ldg(Wa + ((en >> 16) & 0x7FFFu));
+                if (en >> 31) w = -w;
+                ldk<T, K>(xr + (int64_t)(en & 0xFFFFu) * K, xv);
 #pragma unroll
-                    for (int q = 0; q < K; ++q) part[q] = fma(w, xv[q], part[q]);
-                }
-                if (ep >> 31) {
+                for (int q = 0; q < K; ++q) part[q] = fma(w, xv[q], part[q]);
+            }
+            if (J.w >> 31) {
 #pragma unroll
-                    for (int q = 0; q < K; ++q) acc[q] -= part[q];
-                } else {
+                for (int q = 0; q < K; ++q) acc[q] -= part[q];
+            } else {
 #pragma unroll
-                    for (int q = 0; q < K; ++q) acc[q] += part[q];
-                }
+                for (int q = 0; q < K; ++q) acc[q] += part[q];
             }
         }
     }
@@ -217,14 +226,15 @@ __global__ void __launch_bounds__(NT) hx_fused_kernel(HxArgs A, const T *__restr
 template <typename T, int K>
 cudaError_t launch(const Device &Dv, const DevCoefs<T> &C, const T *x, T *y, cudaStream_t s)
 {
-    HxArgs A{Dv.tasks, Dv.blocks, Dv.links, Dv.pp_ptr, Dv.nn_ptr, Dv.p1_ptr, Dv.n1_ptr,
-             Dv.pp_src, Dv.nn_src, Dv.p1_ent, Dv.n1_ent, Dv.llinks, Dv.ppx_ptr, Dv.nnx_ptr, Dv.ppx_src, Dv.nnx_src};
+    HxArgs A{Dv.tasks, Dv.blocks, Dv.pp_ptr, Dv.nn_ptr, Dv.n1_ptr,
+             Dv.pp_src, Dv.nn_src, Dv.n1_ent, Dv.jumps, Dv.jump_ptr, Dv.llinks, Dv.ppx_ptr, Dv.nnx_ptr, Dv.ppx_src, Dv.nnx_src};
     auto run = [&](auto nt) {
         constexpr int NT = decltype(nt)::value;
         hx_fused_kernel<T, K, NT><<<Dv.ntasks, NT, 0, s>>>(A, C.pp_coef, C.nn_coef, C.wpn, C.ppx_coef, C.nnx_coef, x, y);
     };
     // Threads by the number of CTAs: with few, more groups shorten each thread's chain of loads; with many, they only
-    // take registers.  us at 128 / 256 / 512 threads: sd 2p2n (66 CTAs) FP64 k = 1 17 / 15 / 16; sd 4p4n (495) FP32
+    // take registers.  us at 128 / 256 / 512 threads (with the pn links walked one by one; the flat jump lists take
+    // a third off the small ones): sd 2p2n (66 CTAs) FP64 k = 1 17 / 15 / 16; sd 4p4n (495) FP32
     // k = 4 51 / 37 / 34, k = 8 64 / 47 / 49, FP64 k = 8 297 / 254 / 293; pf 3p3n (2,200) k = 1 111 / 98 / 130,
     // k = 4 126 / 154 / 152, k = 8 228 / 219 / 249; pf 4p3n (9,500) k = 1 398 / 413 / 585.
     constexpr bool wide = K * sizeof(T) == 64;

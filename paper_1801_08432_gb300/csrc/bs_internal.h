@@ -388,7 +388,13 @@ struct DevTask {            // one CTA: destination block, proton row, column ti
     int block;
     int row;
     int col0;
-    int pad;
+    int list;               // the row's proton jumps: jump_ptr[list], of every link of its block
+};
+
+struct RowJump {            // a proton one-body jump into a row, with its link
+    int64_t xoff;           // first basis index of the source row
+    uint32_t nptr;          // the link's neutron class in n1_ptr
+    uint32_t w;             // W row of the jump's operator in wpn (at most 64^4 elements) | sign << 31
 };
 
 template <typename T>
@@ -411,6 +417,8 @@ struct Device {
     int64_t *ppx_ptr = nullptr, *nnx_ptr = nullptr;
     int32_t *ppx_src = nullptr, *nnx_src = nullptr;
     DevTask *tasks = nullptr;
+    RowJump *jumps = nullptr;
+    int64_t *jump_ptr = nullptr;
     int ntasks = 0;
     int tile = 0;
     int64_t *pp_ptr = nullptr, *nn_ptr = nullptr;
