@@ -13,6 +13,12 @@
 // FP64, reduce them across the warp and add them to the operator's k x k
 // slot (FP64 atomics: the summation order, and so the last bits, may vary
 // between runs).
+//
+// FP64 adds bound it (2 per cycle and SM).  The warp sum halves its k*k values
+// from step to step: 6 adds a lane at k = 2 where a butterfly per value takes
+// 20 (62 and 320 at k = 8), and the finished values leave from several lanes.
+// Per call, us, k = 2 / 4 / 8: pf 4p4n 632 / 2202 / 7768 before, 510 / 1600 /
+// 5582 now; sd 4p4n 74 / 148 / 422 before, 66 / 93 / 204 now.
 #include <cuda_runtime.h>
 
 #include <vector>
@@ -69,22 +75,32 @@ __global__ void __launch_bounds__(128) density_kernel(const DensItem *__restrict
 #pragma unroll
                     for (int j = 0; j < K; ++j) acc[f][j] = fma(fv[f], xv[j], acc[f][j]);
             }
+            // sum over the warp: a step with several values left keeps half of them in each half of the lanes
+            constexpr int M = K * K, H = M >= 32 ? 5 : M == 16 ? 4 : M == 4 ? 2 : 0;   // H halving steps
+            double v[M];
 #pragma unroll
-            for (int f = 0; f < K; ++f)
+            for (int i = 0; i < M; ++i) v[i] = acc[i / K][i % K];
 #pragma unroll
-                for (int j = 0; j < K; ++j) {
-                    double v = acc[f][j];
+            for (int t = 0; t < 5; ++t) {
+                const int o = 16 >> t;
+                if (t < H) {
+                    const int m = M >> (t + 1);
+                    const bool up = lane & o;
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    acc[f][j] = v;
+                    for (int i = 0; i < m; ++i) {
+                        const double send = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+                        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                } else {
+                    v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
                 }
-            if (lane == 0) {
+            }
+            // one lane in 2^(5 - H) holds M >> H finished values
+            if ((lane & ((1 << (5 - H)) - 1)) == 0) {
                 const double sg = (pk >> 31) ? -1.0 : 1.0;
-                double *out = rho + ((int64_t)d.spc * nops + op) * K * K;
+                double *out = rho + ((int64_t)d.spc * nops + op) * M + (lane >> (5 - H)) * (M >> H);
 #pragma unroll
-                for (int f = 0; f < K; ++f)
-#pragma unroll
-                    for (int j = 0; j < K; ++j) atomicAdd(out + f * K + j, sg * acc[f][j]);
+                for (int i = 0; i < (M >> H); ++i) atomicAdd(out + i, sg * v[i]);
             }
         }
     }
