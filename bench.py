@@ -326,12 +326,12 @@ def lanczos_check(ctx, N, I, torch, stream):
 KERNEL_SOURCES = {1: "bs_hx.cu", 2: "bs_hx_row.cu", 3: "bs_hx_row.cu", 4: "bs_hx_row.cu", 5: "bs_hx_row.cu",
                   6: "bs_hx_pipe.cu", 7: "bs_hx_pipe.cu", 8: "bs_hx_pipe.cu", 9: "bs_hx_pipe.cu", 10: "bs_hx_pipe.cu",
                   11: "bs_hx_core.cu", 12: "bs_hx_core.cu", 13: "bs_hx_core.cu", 14: "bs_hx_core.cu",
-                  15: "bs_hx_core.cu", 16: "bs_hx_core.cu", 17: "bs_hx_core.cu", 18: "bs_hx_core.cu",
+                  15: "bs_hx_core.cu", 16: "bs_hx_pair.cu", 17: "bs_hx_core.cu", 18: "bs_hx_core.cu",
                   19: "bs_hx_core.cu", 20: "bs_hx_core.cu"}
-# ncu summaries of the dominant kernel per mode (the pn-core kernel in 11..20)
+# ncu summaries of the dominant kernel per mode (the pn-core kernel in 11..20 but 16)
 PROFILES = {1: "hx_fused_pf4p4n_k8.md", 2: "hx_row_pf4p4n_k8.md", 6: "hx_pipe_pf4p4n_k8.md",
             11: "hx_core_pf4p4n_k8.md", 12: "hx_core_pf4p4n_k8.md", 13: "hx_core_pf4p4n_k8.md",
-            14: "hx_core_pf4p4n_k8.md", 15: "hx_core_pf4p4n_k8.md", 16: "hx_core_pf4p4n_k8.md",
+            14: "hx_core_pf4p4n_k8.md", 15: "hx_core_pf4p4n_k8.md",
             17: "hx_core_pf4p4n_k8.md", 18: "hx_core_pf4p4n_k8.md", 19: "hx_core_pf4p4n_k8.md",
             20: "hx_core_pf4p4n_k8.md"}
 
@@ -340,8 +340,8 @@ def launches_per_product(mode):
     """Kernels one H x launches in a kernel mode: the core-grouped modes run the
     pn kernel (and in 13 to 16 and 18 to 20 the pp kernel) and the like-particle
     kernel; the row-tile like-particle kernel of 13 to 16, 19 and 20 also adds the
-    partial vectors, the pipelined one of 11, 12, 17 and 18 is followed by the
-    ordered sum; every other mode is one kernel."""
+    partial vectors, that of 18 and the pipelined one of 11, 12 and 17 are
+    followed by the ordered sum; every other mode is one kernel."""
     return {11: 3, 12: 3, 13: 3, 14: 3, 15: 3, 16: 3, 17: 3, 18: 4, 19: 3, 20: 3}.get(mode, 1)
 
 
@@ -367,8 +367,8 @@ def fe52_product(N, I, torch, device, mode=18, nrep=3):
     """The largest workload (pf 6p6n M=0, 52Fe, dim 109,954,620) at its block
     size k = 4: set-up (basis, decoupling, tables, upload) timed on the host,
     then one warm-up and nrep timed FP32 block products H X in the
-    core-grouped mode the autotuner picks for its wide neutron sectors (the
-    pipelined nn kernel after the pp-core kernel), CUDA events around each product and around its
+    core-grouped mode the autotuner picks for its wide neutron sectors (nn by
+    three-row tiles after the pp-core kernel), CUDA events around each product and around its
     pn-core kernel.  Reported beside the main line, not part of its value."""
     orbits, spe, tb = I.space("pf")
     t0 = time.time()

@@ -180,10 +180,12 @@ int bs_apply_H_host_async(bs_ctx *ctx, const void *x_host, void *y_host, int k,
  * the derivative of the pairing gy . H x -- with x = gy = psi (normalized) it
  * is the Hellmann-Feynman derivative dE/dtheta_t, the paper's "diagonal"
  * two-body density X_J(ab,cd) = dE/dV_J(ab,cd) for a TBME slot.  H is linear
- * in theta, so the transition densities gy . x over all jumps (pp and nn per
- * jump, pn per pair of decoupled operators; GPU kernels, FP64 accumulation)
- * are contracted on the host with dW/dtheta, built once per label set by
- * decoupling unit interactions.  x, gy, gx: distinct except x may equal gy.
+ * in theta, so its transition densities (GPU kernels; FP64 or double-float
+ * accumulation: for plain bases of at most 32 states per species one Gram
+ * matrix over pairs per pair key, else one value per jump, and per pair of
+ * decoupled operators for pn) are contracted on the host with dW/dtheta, one
+ * flat list built once per label set.  The first call per loaded interaction
+ * lays out its work units.  x, gy, gx: distinct except x may equal gy.
  * Synchronizes the stream when gtheta != NULL.  Errors: as bs_apply_H,
  * BS_ENOMEM. */
 int bs_apply_H_backward(bs_ctx *ctx, const void *x, const void *gy, void *gx, double *gtheta, int k,
@@ -415,8 +417,9 @@ int bs_debug_eigh_banded(int n, int bw, const double *A, int nval, double *w, do
  * columns); in 13..16 and 18..20 a second persistent kernel computes the pp
  * two-body term per
  * (Z-2)-proton core into C(Z,2) more and a row-tile kernel (4 rows per CTA,
- * 2 in 19 and 20, column tiles of 576 for wider sectors; 18: the first pipelined
- * variant that fits) the nn term and the proton single-particle energies
+ * 2 in 19 and 20, column tiles of 576 for wider sectors; 18: 3 or 2, whichever
+ * fits first, into one more partial vector, else the first pipelined variant
+ * that fits) the nn term and the proton single-particle energies
  * into one more (16 with k = 1, 2: panels of x in shared memory for
  * both like-particle terms, which add the partial vectors);
  * a last kernel
@@ -425,9 +428,11 @@ int bs_debug_eigh_banded(int n, int bw, const double *A, int nval, double *w, do
  * bs_lanczos before it captures a graph; a first call inside a stream
  * capture without it falls back to another kernel).  A mode that does not fit
  * the basis falls back to the tiled kernel.  0 (default) = the mode bs_autotune picked
- * for the call's (k, dtype), else for FP32 one by the size of the basis (16
- * or 20 for large ones, where they apply), else the first pipelined variant,
- * else the first row variant.  All modes give the same result up to summation order.
+ * for the call's (k, dtype), else one by the size of the basis: for FP64 and
+ * W-truncated bases 1 below 50,000 states, else the first pipelined variant,
+ * else the first row variant; for FP32 1 for small ones and narrow neutron
+ * sectors, else 16 (k up to 4) or 20 (k = 8) where they apply, then 13, then
+ * as for FP64.  All modes give the same result up to summation order.
  * Errors: BS_EINVAL. */
 int bs_set_kernel(bs_ctx *ctx, int mode);
 
