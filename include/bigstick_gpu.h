@@ -43,6 +43,10 @@
  *     staging buffers).  Issue them on one stream, or order them with
  *     events: two such calls running at the same time on the GPU race.
  *     bs_apply_H_host_async orders its own products among themselves.
+ *     A captured call keeps the tables and the workspace it was captured
+ *     with: its graph may be replayed until the next bs_build_basis*,
+ *     bs_load_interaction or bs_destroy (a workspace that a later call
+ *     outgrows stays allocated until then).
  */
 #ifndef BIGSTICK_GPU_H
 #define BIGSTICK_GPU_H

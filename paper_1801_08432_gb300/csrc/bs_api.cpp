@@ -422,6 +422,7 @@ void bs_destroy(bs_ctx *c)
             if (c->hxa_free[i]) cudaEventDestroy(c->hxa_free[i]);
         }
         if (c->hxa_prod) cudaEventDestroy(c->hxa_prod);
+        release_hx_old(c);
         if (c->core_part) cudaFree(c->core_part);
         for (cudaEvent_t ev : c->tev) cudaEventDestroy(ev);
     }
@@ -435,7 +436,10 @@ int bs_build_basis_trunc(bs_ctx *c, const bs_orbit *orbits, int n_orbits, int Z,
 {
     return guarded(c, [&]() -> int {
         c->have_basis = c->have_int = false;
-        if (c->device >= 0) release(c->dev);
+        if (c->device >= 0) {
+            release(c->dev);
+            release_hx_old(c);
+        }
         if (max_excite < -1) { c->err = "build_basis: max_excite must be -1 (no truncation) or >= 0"; return BS_EINVAL; }
         int rc = build_basis(c->basis, orbits, n_orbits, Z, N, twoM, parity, max_excite, c->err);
         if (rc) return rc;
@@ -517,6 +521,7 @@ int bs_load_interaction(bs_ctx *c, const double *spe, int n_spe, const bs_tbme *
         rc = build_tables(c->basis, c->inter, c->tab, c->err, nsm);
         if (rc) return rc;
         if (c->device >= 0) {
+            release_hx_old(c);
             release_adj(c->adj);
             if (c->adj_gpp) { cudaFree(c->adj_gpp); cudaFree(c->adj_gnn); cudaFree(c->adj_rho); }
             c->adj_gpp = c->adj_gnn = c->adj_rho = nullptr;

@@ -1037,9 +1037,11 @@ int prepare_hx(const bs_ctx *c, int k, bs_dtype dt, std::string &err)
 {
     const size_t need = core_applies(c, k, dt) ? part_bytes(c, k) : pair_applies(c, k, dt) ? pair_bytes(c, k) : 0;
     if (c->core_part_bytes >= need) return BS_OK;
-    if (c->core_part) cudaFree(c->core_part);
+    if (c->core_part && c->core_part_captured) c->core_part_old.push_back(c->core_part);
+    else if (c->core_part) cudaFree(c->core_part);
     c->core_part = nullptr;
     c->core_part_bytes = 0;
+    c->core_part_captured = false;
     cudaError_t e = cudaMalloc(&c->core_part, need);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
@@ -1049,6 +1051,14 @@ int prepare_hx(const bs_ctx *c, int k, bs_dtype dt, std::string &err)
     }
     c->core_part_bytes = need;
     return BS_OK;
+}
+
+// Outgrown buffers: freed with the tables, without which no captured product can be replayed either.
+void release_hx_old(const bs_ctx *c)
+{
+    for (void *p : c->core_part_old) cudaFree(p);
+    c->core_part_old.clear();
+    c->core_part_captured = false;
 }
 
 // Core-grouped pn kernel variant v followed by the pipelined like-particle
@@ -1066,13 +1076,14 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
         const cudaError_t pe = launch_hx_pair(c, nullptr, nullptr, k, s, ok);
         if (pe != cudaSuccess || !ok) return pe;
     }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t ce = cudaStreamIsCapturing(s, &cap);
+    if (ce != cudaSuccess) return ce;
     if (c->core_part_bytes < (core ? part_bytes(c, k) : pair_bytes(c, k))) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        cudaError_t e = cudaStreamIsCapturing(s, &cap);
-        if (e != cudaSuccess) return e;
         std::string err;
         if (cap != cudaStreamCaptureStatusNone || prepare_hx(c, k, dt, err) != BS_OK) return cudaSuccess;
     }
+    if (cap != cudaStreamCaptureStatusNone) c->core_part_captured = true;
     if (!core) {
         cudaError_t e;
         if (t0 && (e = cudaEventRecord(t0, s)) != cudaSuccess) return e;

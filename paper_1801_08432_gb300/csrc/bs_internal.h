@@ -500,6 +500,10 @@ struct bs_ctx {
     // partial sums of the core-grouped pn kernel: nz x dim x k elements, grown on demand
     mutable void *core_part = nullptr;
     mutable size_t core_part_bytes = 0;
+    // a caller's graph may hold the buffer's address: then a larger one does not free it, it is kept until the
+    // tables that the graph also holds go (or the context)
+    mutable bool core_part_captured = false;
+    mutable std::vector<void *> core_part_old;
     // event pairs around the dominant kernel of each product (bs_time_kernel)
     std::vector<cudaEvent_t> tev;
     mutable int tev_used = 0;
@@ -557,4 +561,5 @@ int pipe_variants();
 int core_variants();
 // allocates what launch_hx needs for (k, dtype) outside any stream capture
 int prepare_hx(const bs_ctx *ctx, int k, bs_dtype dt, std::string &err);
+void release_hx_old(const bs_ctx *ctx);
 }  // namespace bs

@@ -2088,6 +2088,12 @@ int run_lanczos(bs_ctx *c, const bs_lanczos_opts &o_in, const void *pivot, doubl
         std::string ignored;
         (void)prepare_hx(c, o.k, o.dtype, ignored);
     }
+    // this call's own graph does not outlive it
+    struct Captured {
+        const bs_ctx *c;
+        bool before;
+        ~Captured() { c->core_part_captured = before; }
+    } captured{c, c->core_part_captured};
     if (o.dtype == BS_F64) {
         switch (o.k) {
         case 1: return lanczos_run<double, 1>(c, o, pivot, evals, evecs, rep, sreq);
