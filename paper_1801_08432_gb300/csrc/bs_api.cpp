@@ -436,6 +436,7 @@ int bs_build_basis_trunc(bs_ctx *c, const bs_orbit *orbits, int n_orbits, int Z,
 {
     return guarded(c, [&]() -> int {
         c->have_basis = c->have_int = false;
+        c->have_dW = false;   // its indices are those of the former basis' tables
         if (c->device >= 0) {
             release(c->dev);
             release_hx_old(c);
@@ -508,7 +509,7 @@ int bs_load_interaction(bs_ctx *c, const double *spe, int n_spe, const bs_tbme *
             for (size_t i = 0; same_labels && i < tb.size(); ++i)
                 same_labels = tb[i].a == c->tbme_in[i].a && tb[i].b == c->tbme_in[i].b && tb[i].c == c->tbme_in[i].c &&
                               tb[i].d == c->tbme_in[i].d && tb[i].J == c->tbme_in[i].J && tb[i].T == c->tbme_in[i].T;
-            if (!same_labels) c->have_dW = false;   // derivative tables depend on the labels only
+            if (!same_labels) c->have_dW = false;   // on one basis the derivative tables depend on the labels only
             c->spe_in.assign(spe, spe + n_spe);
             c->tbme_in.swap(tb);
         }
