@@ -904,14 +904,36 @@ __device__ __forceinline__ void df_fma2(float2 &hi, float2 &lo, float2 a, float2
     hi = t;
 }
 
+// hi + lo = a b, exactly
+__device__ __forceinline__ void df_prod2(float2 &hi, float2 &lo, float2 a, float2 b, float2 nz)
+{
+    hi = __ffma2_rn(a, b, nz);
+    lo = __ffma2_rn(a, b, make_float2(-hi.x, -hi.y));
+}
+
+// hi + lo += h + l, normalized: the operations of df_sum (x - y as fma(y, -1, x), the same rounding)
+__device__ __forceinline__ void df_sum2(float2 &hi, float2 &lo, float2 h, float2 l)
+{
+    const float2 m = make_float2(-1.0f, -1.0f);
+    const float2 s = __fadd2_rn(hi, h), bb = __ffma2_rn(hi, m, s);
+    const float2 e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bb, m, s), m, hi), __ffma2_rn(bb, m, h));
+    const float2 t = __fadd2_rn(__fadd2_rn(e, lo), l);
+    hi = __fadd2_rn(s, t);
+    lo = __ffma2_rn(__ffma2_rn(s, m, hi), m, t);
+}
+
 // V_b^T W for FP32 blocks with exact products (partial layout as rs_dots).
 // Block by block: a CTA streams the tiles b of V and W of all its chunks in
 // pairs through one ring, so that a block's sums stay in registers
 // (double-float, thread (r, i): V column i, rows r + (256 / K) m) over all of
 // them and lanes and warps are combined once per block instead of once per
-// tile; W comes from L2 from the second block on.  Bound by FP32 issue, 8
-// operations per product: 48Cr k = 8, 24 blocks 1.97 ms -> 0.90 ms (HBM floor
-// 0.23 ms).
+// tile; W comes from L2 from the second block on.  A tile's eight rows are
+// summed by themselves and joined to the running sums normalized: a remainder
+// lo that only grows over all tiles loses 10 bits at 1,500 products a thread
+// (equal products, by emulation: 2^-31.9 of the sum against 2^-42.6).  Bound
+// by FP32 issue, 70 packed operations per eight products and pair: 48Cr
+// k = 8, 24 blocks 1.97 ms by rs_dots, 0.90 ms this way without the joins,
+// which add 0.06 ms (HBM floor 0.23 ms).
 constexpr int kRxS = 5;   // ring stages of two tiles: 80 KB, two CTAs on an SM
 
 template <int K>
@@ -980,15 +1002,19 @@ __global__ void __launch_bounds__(kRsCons + 32, 2)
             const int rows = (int)(min((int64_t)kRsCE, nel - ch * kRsCE) / K);
             const float *tv = ring + (size_t)q.s * 2 * kRsCE, *tw = tv + kRsCE;
             if (!bad) {
+                float2 th[NP], tl[NP];   // this tile's sums
                 if constexpr (K == 1) {
 #pragma unroll
                     for (int m = 0; m < kRsRT; m += 2) {
                         const int a = r + NR * m, c = a + NR;
                         const float2 v = make_float2(a < rows ? tv[a] : 0.f, c < rows ? tv[c] : 0.f);
                         const float2 w = make_float2(a < rows ? tw[a] : 0.f, c < rows ? tw[c] : 0.f);
-                        df_fma2(hi[0], lo[0], v, w, nz);
+                        if (m == 0) df_prod2(th[0], tl[0], v, w, nz);
+                        else df_fma2(th[0], tl[0], v, w, nz);
                     }
                 } else {
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) th[p] = tl[p] = make_float2(0.f, 0.f);
 #pragma unroll
                     for (int m = 0; m < kRsRT; ++m) {
                         const int a = r + NR * m;
@@ -997,11 +1023,16 @@ __global__ void __launch_bounds__(kRsCons + 32, 2)
                             float w[K];
                             ldrow<float, K>(tw + a * K, w);
 #pragma unroll
-                            for (int p = 0; p < NP; ++p)
-                                df_fma2(hi[p], lo[p], make_float2(v, v), make_float2(w[2 * p], w[2 * p + 1]), nz);
+                            for (int p = 0; p < NP; ++p) {
+                                const float2 vv = make_float2(v, v), ww = make_float2(w[2 * p], w[2 * p + 1]);
+                                if (m == 0) df_prod2(th[p], tl[p], vv, ww, nz);
+                                else df_fma2(th[p], tl[p], vv, ww, nz);
+                            }
                         }
                     }
                 }
+#pragma unroll
+                for (int p = 0; p < NP; ++p) df_sum2(hi[p], lo[p], th[p], tl[p]);
             }
             __syncwarp();
             if (lane == 0) bar_arrive(empty0 + 8u * q.s);
