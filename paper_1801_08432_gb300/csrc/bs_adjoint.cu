@@ -14,9 +14,12 @@
 // adj_gram.  Spaces its tables do not cover (more than 32 states per
 // species) take the kernels before it: one value per pp and nn jump, split
 // into two-body moves on the host, and the pn densities by atomics per pair
-// of jumps.  Products of FP32 vectors are formed in FP32; their sums carry
-// 48 bits or more, and are collected with FP64 atomics (the order of those
-// additions, and so the last bits, may differ from run to run).
+// of jumps.  Products of FP32 vectors are formed in FP32.  adj_gram sums a
+// unit's columns in double-float, normalized every 8 to 15 columns of a
+// thread (each time within 135 2^-48 of the sum of magnitudes; the products
+// themselves are rounded by 2^-24).  Everything else is FP64, collected with
+// FP64 atomics (the order of those additions, and so the last bits, may
+// differ from run to run).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -264,7 +267,7 @@ struct GramSum<double> {
     }
     using Part = double;
     __device__ __forceinline__ double part(int i) const { return v[i]; }
-    static __device__ __forceinline__ double join(double a, double b) { return a + b; }
+    __device__ __forceinline__ void normalize() {}
     static __device__ __forceinline__ double value(double a) { return a; }
 };
 template <>
@@ -280,12 +283,24 @@ struct GramSum<float> {
         hi = t;
     }
     __device__ __forceinline__ void add_prod(float a0, float a1, float b) { add(__fmul_rn(a0, b), __fmul_rn(a1, b)); }
+    // lo back below the last bit of hi: the remainders that add collects are rounded to lo's last bit
+    __device__ __forceinline__ void normalize()
+    {
+        const float2 m = make_float2(-1.0f, -1.0f), t = __fadd2_rn(hi, lo);
+        lo = __ffma2_rn(__ffma2_rn(hi, m, t), m, lo);
+        hi = t;
+    }
     using Part = float2;   // hi, lo
     __device__ __forceinline__ float2 part(int i) const { return i ? make_float2(hi.y, lo.y) : make_float2(hi.x, lo.x); }
     static __device__ __forceinline__ float2 join(float2 a, float2 b)
     {
         const float t = a.x + b.x, z = t - a.x;
         return make_float2(t, a.y + b.y + ((a.x - (t - z)) + (b.x - z)));
+    }
+    static __device__ __forceinline__ float2 normal(float2 a)
+    {
+        const float t = a.x + a.y;
+        return make_float2(t, a.y - (t - a.x));
     }
     static __device__ __forceinline__ double value(float2 a) { return (double)a.x + (double)a.y; }
 };
@@ -384,6 +399,7 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
         }
         __syncthreads();
         GramSum<T> acc[2][RB];
+        int n = 0;   // columns since the sums were normalized
         for (int c0 = 0; c0 < U.ncol; c0 += CH) {
             if (c0) __syncthreads();
             // columns first, then elements: NB dependent pairs of loads in flight
@@ -442,28 +458,38 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
             __syncthreads();
             const int cn = min(CH, U.ncol - c0);
             if (slice < S) {
-                for (int c = slice; c < cn; c += S) {
-                    alignas(16) T a[4][K], b[RB][K];
+                for (int cb = slice; cb < cn; cb += 8 * S) {
+                    const int ce = min(cn, cb + 8 * S);
+                    for (int c = cb; c < ce; c += S, ++n) {
+                        alignas(16) T a[4][K], b[RB][K];
 #pragma unroll
-                    for (int p = 0; p < 4; ++p) gget<T, K>(sg + (ia + ga * p) * LD + c * K, a[p]);
+                        for (int p = 0; p < 4; ++p) gget<T, K>(sg + (ia + ga * p) * LD + c * K, a[p]);
 #pragma unroll
-                    for (int q = 0; q < RB; ++q) gget<T, K>(sx + (ib + gb * q) * LD + c * K, b[q]);
+                        for (int q = 0; q < RB; ++q) gget<T, K>(sx + (ib + gb * q) * LD + c * K, b[q]);
 #pragma unroll
-                    for (int p = 0; p < 2; ++p)
+                        for (int p = 0; p < 2; ++p)
 #pragma unroll
-                        for (int q = 0; q < RB; ++q) {
-                            if constexpr (K == 1) {
-                                acc[p][q].add_prod(a[2 * p][0], a[2 * p + 1][0], b[q][0]);
-                            } else {
-                                T f0 = a[2 * p][0] * b[q][0], f1 = a[2 * p + 1][0] * b[q][0];
+                            for (int q = 0; q < RB; ++q) {
+                                if constexpr (K == 1) {
+                                    acc[p][q].add_prod(a[2 * p][0], a[2 * p + 1][0], b[q][0]);
+                                } else {
+                                    T f0 = a[2 * p][0] * b[q][0], f1 = a[2 * p + 1][0] * b[q][0];
 #pragma unroll
-                                for (int k = 1; k < K; ++k) {
-                                    f0 = fma(a[2 * p][k], b[q][k], f0);
-                                    f1 = fma(a[2 * p + 1][k], b[q][k], f1);
+                                    for (int k = 1; k < K; ++k) {
+                                        f0 = fma(a[2 * p][k], b[q][k], f0);
+                                        f1 = fma(a[2 * p + 1][k], b[q][k], f1);
+                                    }
+                                    acc[p][q].add(f0, f1);
                                 }
-                                acc[p][q].add(f0, f1);
                             }
-                        }
+                    }
+                    if (n >= 8) {   // (not tested column by column: that costs 45 us of 48Cr k = 4)
+                        n = 0;
+#pragma unroll
+                        for (int p = 0; p < 2; ++p)
+#pragma unroll
+                            for (int q = 0; q < RB; ++q) acc[p][q].normalize();
+                    }
                 }
             }
         }
@@ -485,7 +511,18 @@ __global__ void __launch_bounds__(kGramThreads, 2) adj_gram(GramArgs A, const T 
                 const int a = th % ga + ga * (pq / RB), b = th / ga + gb * (pq % RB);
                 if (a >= U.na || b >= U.nb) continue;
                 Part v = part[pq * kGramThreads + th];
-                for (int sl = 1; sl < S; ++sl) v = GramSum<T>::join(v, part[pq * kGramThreads + sl * nt + th]);
+                if constexpr (std::is_same<T, double>::value) {
+                    for (int sl = 1; sl < S; ++sl) v += part[pq * kGramThreads + sl * nt + th];
+                } else {
+                    for (int s0 = 1; s0 < S; s0 += 8) {   // eight loads under way (one by one: 130 us more at 48Cr k = 4)
+                        Part w[8];
+#pragma unroll
+                        for (int h = 0; h < 8; ++h) w[h] = s0 + h < S ? part[pq * kGramThreads + (s0 + h) * nt + th] : Part{};
+#pragma unroll
+                        for (int h = 0; h < 8; ++h) v = GramSum<T>::join(v, w[h]);
+                        v = GramSum<T>::normal(v);
+                    }
+                }
                 mat[rp[na + b] * kGramTile + rp[a]] += GramSum<T>::value(v);
             }
         } else if (slice < S) {
