@@ -189,7 +189,9 @@ int bs_apply_H_host_async(bs_ctx *ctx, const void *x_host, void *y_host, int k,
  * matrix over pairs per pair key, else one value per jump, and per pair of
  * decoupled operators for pn) are contracted on the host with dW/dtheta, one
  * flat list built once per label set.  The first call per loaded interaction
- * lays out its work units.  x, gy, gx: distinct except x may equal gy.
+ * lays out its work units.  Vectors with infinite elements or FP32 sums
+ * beyond 3.4e38 take the kernels by jumps on any basis.
+ * x, gy, gx: distinct except x may equal gy.
  * Synchronizes the stream when gtheta != NULL.  Errors: as bs_apply_H,
  * BS_ENOMEM. */
 int bs_apply_H_backward(bs_ctx *ctx, const void *x, const void *gy, void *gx, double *gtheta, int k,

@@ -12,7 +12,7 @@
 // with the cores (Z-1 protons, N-1 neutrons) for pn, (N-2 neutrons, any
 // proton SD) for nn and (Z-2 protons, any neutron SD) for pp: see
 // adj_gram.  Spaces its tables do not cover (more than 32 states per
-// species) take the kernels before it: one value per pp and nn jump, split
+// species), and vectors that leave its range, take the kernels before it: one value per pp and nn jump, split
 // into two-body moves on the host, and the pn densities by atomics per pair
 // of jumps.  Products of FP32 vectors are formed in FP32.  adj_gram sums a
 // unit's columns in double-float, normalized every 8 to 15 columns of a
@@ -214,8 +214,13 @@ int launch_adj(bs_ctx *c, const T *x, const T *gy, cudaStream_t s, std::vector<i
     adj_pp<T, K><<<D.nrtasks, 128, 0, s>>>(D.rtasks, D.blocks, D.pp_ptr, D.pp_src, x, gy, c->adj_gpp);
     if (!cb.empty()) {
         int *dcb = nullptr, *dcl = nullptr;
-        cudaMallocAsync((void **)&dcb, cb.size() * sizeof(int), s);
-        cudaMallocAsync((void **)&dcl, cl.size() * sizeof(int), s);
+        cudaError_t me = cudaMallocAsync((void **)&dcb, cb.size() * sizeof(int), s);
+        if (me == cudaSuccess && (me = cudaMallocAsync((void **)&dcl, cl.size() * sizeof(int), s)) != cudaSuccess) cudaFreeAsync(dcb, s);
+        if (me != cudaSuccess) {
+            (void)cudaGetLastError();
+            c->err = std::string("adjoint: ") + cudaGetErrorString(me);
+            return BS_ENOMEM;
+        }
         cudaMemcpyAsync(dcb, cb.data(), cb.size() * sizeof(int), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(dcl, cl.data(), cl.size() * sizeof(int), cudaMemcpyHostToDevice, s);
         adj_nn<T, K><<<(int)cb.size(), 128, 0, s>>>(D.blocks, dcb, dcl, D.nn_ptr, D.nn_src, x, gy, c->adj_gnn);
@@ -818,8 +823,8 @@ int build_plan(bs_ctx *c)
     return BS_OK;
 }
 
-// gtheta from the Gram matrices
-int gram_backward(bs_ctx *c, const void *x, const void *gy, double *gtheta, int k, bs_dtype dt, cudaStream_t s)
+// gtheta from the Gram matrices; nothing is added where they are not all finite
+int gram_backward(bs_ctx *c, const void *x, const void *gy, double *gtheta, int k, bs_dtype dt, cudaStream_t s, bool &finite)
 {
     AdjPlan &P = c->adj;
     const Interaction &I = c->inter;
@@ -842,6 +847,8 @@ int gram_backward(bs_ctx *c, const void *x, const void *gy, double *gtheta, int 
         c->err = std::string("adjoint: ") + cudaGetErrorString(e);
         return BS_ECUDA;
     }
+    finite = std::all_of(P.host, P.host + P.nout, [](double v) { return std::isfinite(v); });
+    if (!finite) return BS_OK;
     const int ns = (int)B.st.size(), no = (int)c->spe_in.size();
     std::vector<double> n1((size_t)ns, 0.0);
     for (int spc = 0; spc < 2; ++spc) {
@@ -884,7 +891,13 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
         c->have_dW = true;
     }
     if (!c->adj.tried && (rc = build_plan(c))) return rc;
-    if (c->adj.on) return gram_backward(c, x, gy, gtheta, k, dt, s);
+    if (c->adj.on) {
+        // A sum of FP32 products beyond 3.4e38 leaves double-float's range, and an infinite element meets the zeros that
+        // stand for occupied states: such vectors take the kernels by jumps, whose sums are FP64 over the jumps alone.
+        bool finite = false;
+        rc = gram_backward(c, x, gy, gtheta, k, dt, s, finite);
+        if (rc || finite) return rc;
+    }
     const Tables &T = c->tab;
     const Interaction &I = c->inter;
     cudaError_t e;
@@ -893,6 +906,10 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
             (e = cudaMalloc(&c->adj_gnn, std::max<size_t>(1, T.nn.src.size()) * sizeof(double))) != cudaSuccess ||
             (e = cudaMalloc(&c->adj_rho, std::max<size_t>(1, I.Wpn.size()) * sizeof(double))) != cudaSuccess) {
             c->err = std::string("adjoint: ") + cudaGetErrorString(e);
+            (void)cudaGetLastError();
+            cudaFree(c->adj_gpp);   // all or none
+            cudaFree(c->adj_gnn);
+            c->adj_gpp = c->adj_gnn = c->adj_rho = nullptr;
             return BS_ENOMEM;
         }
     }
