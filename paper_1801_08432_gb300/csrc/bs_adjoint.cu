@@ -26,6 +26,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <new>
 #include <type_traits>
 
 #include "bs_internal.h"
@@ -665,7 +666,18 @@ cudaError_t put_plan(AdjPlan &P, V *&d, const std::vector<V> &h)
     return h.empty() ? cudaSuccess : cudaMemcpy(d, h.data(), h.size() * sizeof(V), cudaMemcpyHostToDevice);
 }
 
-// Units of the Gram matrices, once per loaded interaction; false (with no error) where they do not apply.
+// No plan: for want of memory the kernels by jumps run until the next load.
+int plan_failed(bs_ctx *c, cudaError_t e)
+{
+    (void)cudaGetLastError();
+    release_adj(c->adj);
+    c->adj.tried = true;
+    if (e == cudaErrorMemoryAllocation) return BS_OK;
+    c->err = std::string("adjoint tables: ") + cudaGetErrorString(e);
+    return BS_ECUDA;
+}
+
+// Units of the Gram matrices, once per loaded interaction; P.on stays false (with no error) where they do not apply.
 int build_plan(bs_ctx *c)
 {
     AdjPlan &P = c->adj;
@@ -681,10 +693,7 @@ int build_plan(bs_ctx *c)
     cudaError_t e;
     P.ncn = R.ncn;
     if ((e = put_plan(P, P.colpos, R.colpos)) != cudaSuccess || (e = put_plan(P, P.nsign, R.nsign)) != cudaSuccess) {
-        c->err = std::string("adjoint tables: ") + cudaGetErrorString(e);
-        (void)cudaGetLastError();
-        release_adj(P);
-        return e == cudaErrorMemoryAllocation ? BS_ENOMEM : BS_ECUDA;
+        return plan_failed(c, e);
     }
     struct U { GramUnit u; double cost; };
     std::vector<U> units;
@@ -814,10 +823,7 @@ int build_plan(bs_ctx *c)
         (e = put_plan(P, P.range, range)) != cudaSuccess || (e = put_plan(P, P.ndtasks, nt)) != cudaSuccess ||
         (e = put_plan(P, P.out, std::vector<double>((size_t)nout + 1, 0.0))) != cudaSuccess ||
         (e = cudaMallocHost((void **)&P.host, (size_t)nout * sizeof(double))) != cudaSuccess) {
-        c->err = std::string("adjoint tables: ") + cudaGetErrorString(e);
-        (void)cudaGetLastError();
-        release_adj(P);
-        return e == cudaErrorMemoryAllocation ? BS_ENOMEM : BS_ECUDA;
+        return plan_failed(c, e);
     }
     P.on = true;
     return BS_OK;
@@ -890,7 +896,14 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
         build_interaction_derivatives(c->basis, c->inter, c->tbme_in, c->dWpp, c->dWpn);
         c->have_dW = true;
     }
-    if (!c->adj.tried && (rc = build_plan(c))) return rc;
+    if (!c->adj.tried) {
+        try {
+            rc = build_plan(c);
+        } catch (const std::bad_alloc &) {
+            rc = plan_failed(c, cudaErrorMemoryAllocation);
+        }
+        if (rc) return rc;
+    }
     if (c->adj.on) {
         // A sum of FP32 products beyond 3.4e38 leaves double-float's range, and an infinite element meets the zeros that
         // stand for occupied states: such vectors take the kernels by jumps, whose sums are FP64 over the jumps alone.

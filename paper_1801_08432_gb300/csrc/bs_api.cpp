@@ -167,6 +167,56 @@ static void make_row_tasks(const Basis &B, const Tables &T, std::vector<RowTask>
     for (size_t i = 0; i < v.size(); ++i) tasks[i] = v[i].t;
 }
 
+// Tables of the pair-core product; nothing where no proton core's rows fit the kernel.
+int upload_pair(const Basis &B, const Tables &T, Device &D, std::string &err)
+{
+    const PairTables &R = T.pair;
+    int rc;
+    for (int v = 0; v < 3; ++v) {
+        const int cap = pair_cap_cols(4 >> v, R.max_rec);
+        if (v > 0 && D.pr[v - 1].nitems && D.pr[v - 1].cols >= R.max_cols) { D.pr[v] = D.pr[v - 1]; continue; }
+        PairItems O;
+        // a proton core's rows all at once, or this many components are not taken together: every
+        // part of its rows would gather all of x again
+        if (cap < R.max_cols || !build_pair_items(R, cap, O)) continue;
+        Device::PairDev &q = D.pr[v];
+        if ((rc = put(D, q.items, O.items.data(), O.items.size(), err))) return rc;
+        if ((rc = put(D, q.tiles, O.tiles.data(), O.tiles.size(), err))) return rc;
+        if ((rc = put(D, q.rows, O.rows.data(), O.rows.size(), err))) return rc;
+        if ((rc = put(D, q.store, O.store.data(), O.store.size(), err))) return rc;
+        q.nitems = (int)O.items.size();
+        q.cols = O.max_cols;
+        q.max_tiles = O.max_tiles;
+        q.max_rows = O.max_rows;
+        q.max_rec = O.max_rec;
+    }
+    if (!D.pr[0].nitems && !D.pr[1].nitems && !D.pr[2].nitems) return BS_OK;
+    D.pr_ncn = R.ncn;
+    if ((rc = put(D, D.pr_colpos, R.colpos.data(), R.colpos.size(), err))) return rc;
+    if ((rc = put(D, D.pr_nsign, R.nsign.data(), R.nsign.size(), err))) return rc;
+    const std::vector<float> f = cast<float>(R.w);
+    if ((rc = put(D, D.pr_w, f.data(), f.size(), err))) return rc;
+    if ((rc = put(D, D.pr_recs, R.recs.data(), R.recs.size(), err))) return rc;
+    for (int spc = 0; spc < 2; ++spc) {   // like-particle panels
+        Device::LikeDev &q = D.like[spc];
+        std::vector<LikePanel> O;
+        build_like_panels(B, spc, 32, O, q.max_n);
+        const int pw = like_panel_width(q.max_n);
+        if (!pw) continue;
+        LikeLists L;
+        build_like_lists(spc ? T.nn : T.pp, L);
+        if ((rc = put(D, q.ptr, L.ptr.data(), L.ptr.size(), err))) return rc;
+        if ((rc = put(D, q.ent, L.ent.data(), L.ent.size(), err))) return rc;
+        for (int v = 0; v < 2; ++v) {
+            build_like_panels(B, spc, pw >> v, O, q.max_n);
+            q.npanels[v] = (int)O.size();
+            if ((rc = put(D, q.panels[v], O.data(), O.size(), err))) return rc;
+        }
+        q.pw = pw;
+    }
+    return BS_OK;
+}
+
 int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std::string &err)
 {
     release(D);
@@ -332,52 +382,28 @@ int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std
         (R == 2 ? D.nnntasks2 : R == 3 ? D.nnntasks3 : D.nnntasks4) = (int)nt.size();
         if ((rc = put(D, dst, nt.data(), nt.size(), err))) return rc;
     }
-    for (int spc = 0; spc < 2 && T.pair.on; ++spc) {   // like-particle panels
-        Device::LikeDev &q = D.like[spc];
-        std::vector<LikePanel> O;
-        build_like_panels(B, spc, 32, O, q.max_n);
-        q.pw = like_panel_width(q.max_n);
-        if (!q.pw) continue;
-        LikeLists L;
-        build_like_lists(spc ? T.nn : T.pp, L);
-        if ((rc = put(D, q.ptr, L.ptr.data(), L.ptr.size(), err))) return rc;
-        if ((rc = put(D, q.ent, L.ent.data(), L.ent.size(), err))) return rc;
-        for (int v = 0; v < 2; ++v) {
-            build_like_panels(B, spc, q.pw >> v, O, q.max_n);
-            q.npanels[v] = (int)O.size();
-            if ((rc = put(D, q.panels[v], O.data(), O.size(), err))) return rc;
-        }
-    }
-    if (T.pair.on) {   // pair-core pn kernel
-        const PairTables &R = T.pair;
-        D.pr_ncn = R.ncn;
-        if ((rc = put(D, D.pr_colpos, R.colpos.data(), R.colpos.size(), err))) return rc;
-        if ((rc = put(D, D.pr_nsign, R.nsign.data(), R.nsign.size(), err))) return rc;
-        f = cast<float>(R.w);
-        if ((rc = put(D, D.pr_w, f.data(), f.size(), err))) return rc;
-        if ((rc = put(D, D.pr_recs, R.recs.data(), R.recs.size(), err))) return rc;
-        for (int v = 0; v < 3; ++v) {
-            const int cap = pair_cap_cols(4 >> v, R.max_rec);
-            if (v > 0 && D.pr[v - 1].nitems && D.pr[v - 1].cols >= R.max_cols) { D.pr[v] = D.pr[v - 1]; continue; }
-            PairItems O;
-            // a proton core's rows all at once, or this many components are not taken together: every
-            // part of its rows would gather all of x again
-            if (cap < R.max_cols || !build_pair_items(R, cap, O)) continue;
-            Device::PairDev &q = D.pr[v];
-            q.nitems = (int)O.items.size();
-            q.cols = O.max_cols;
-            q.max_tiles = O.max_tiles;
-            q.max_rows = O.max_rows;
-            q.max_rec = O.max_rec;
-            if ((rc = put(D, q.items, O.items.data(), O.items.size(), err))) return rc;
-            if ((rc = put(D, q.tiles, O.tiles.data(), O.tiles.size(), err))) return rc;
-            if ((rc = put(D, q.rows, O.rows.data(), O.rows.size(), err))) return rc;
-            if ((rc = put(D, q.store, O.store.data(), O.store.size(), err))) return rc;
-        }
-    }
     f = cast<float>(T.ww);
     if ((rc = put(D, D.ww32, f.data(), f.size(), err))) return rc;
-    return BS_OK;
+    // last and optional: without them the other kernels run
+    const size_t kept = D.owned.size();
+    try {
+        rc = T.pair.on ? upload_pair(B, T, D, err) : BS_OK;
+    } catch (const std::bad_alloc &) {
+        rc = BS_ENOMEM;
+    }
+    if (rc == BS_ENOMEM) {
+        (void)cudaGetLastError();
+        for (size_t n = kept; n < D.owned.size(); ++n) cudaFree(D.owned[n]);
+        D.owned.resize(kept);
+        for (Device::LikeDev &q : D.like) q = Device::LikeDev();
+        for (Device::PairDev &q : D.pr) q = Device::PairDev();
+        D.pr_colpos = nullptr;
+        D.pr_nsign = nullptr;
+        D.pr_w = nullptr;
+        D.pr_recs = nullptr;
+        rc = BS_OK;
+    }
+    return rc;
 }
 
 }  // namespace bs

@@ -14,6 +14,7 @@
 // one CTA.
 #include <algorithm>
 #include <map>
+#include <new>
 #include <tuple>
 
 #include "bs_internal.h"
@@ -171,11 +172,10 @@ void build_pair_tables(const Basis &B, const Interaction &I, PairTables &T, int6
     // ... pair records by neutron group, and output rows
     struct Out { std::vector<PairRec> recs; std::vector<uint8_t> state; std::vector<PairGroup> grps; std::vector<PairRow> rows; };
     std::vector<Out> outs(pcs.size());
-#pragma omp parallel for schedule(dynamic, 16)
-    for (int64_t n = 0; n < (int64_t)pcs.size(); ++n) {
+    auto records = [&](int64_t n) {
         const PC &c = pcs[(size_t)n];
         Out &o = outs[(size_t)n];
-        if (c.order.empty()) continue;
+        if (c.order.empty()) return;
         for (const Group &g : groups) {
             const std::pair<int, int> key{B.twoM - c.key.twoM - g.key.twoM, B.par ^ c.key.par ^ g.key.par};
             auto pit = pairs.find(key);
@@ -218,7 +218,18 @@ void build_pair_tables(const Basis &B, const Interaction &I, PairTables &T, int6
                 R.pad = 0;
                 o.rows.push_back(R);
             }
+    };
+    bool failed = false;   // (no exception may leave the parallel region)
+#pragma omp parallel for schedule(dynamic, 16)
+    for (int64_t n = 0; n < (int64_t)pcs.size(); ++n) {
+        try {
+            records(n);
+        } catch (const std::bad_alloc &) {
+#pragma omp atomic write
+            failed = true;
+        }
     }
+    if (failed) throw std::bad_alloc();
     for (size_t n = 0; n < pcs.size(); ++n) {
         Out &o = outs[n];
         if (o.rows.empty()) continue;

@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <cmath>
 #include <map>
+#include <new>
 #include <numeric>
 
 #include "bs_internal.h"
@@ -1237,7 +1238,11 @@ int build_tables(const Basis &B, const Interaction &I, Tables &T, std::string &e
         T.ops_nn += onn;
     }
     T.ops_per_vector = ops;
-    build_pair_tables(B, I, T.pair, pair_cap_cols(1, 0));
+    try {   // optional, as on the device
+        build_pair_tables(B, I, T.pair, pair_cap_cols(1, 0));
+    } catch (const std::bad_alloc &) {
+        T.pair = PairTables();
+    }
     if (B.trunc) return BS_OK;   // the core-grouped tables assume one neutron sector per proton sector
     {   // the pp-core kernel packs a destination row and its partial rank into one int
         const int Z = B.sp[0].nparticles;
