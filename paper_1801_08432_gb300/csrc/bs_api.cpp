@@ -173,12 +173,11 @@ int upload_pair(const Basis &B, const Tables &T, Device &D, std::string &err)
     const PairTables &R = T.pair;
     int rc;
     for (int v = 0; v < 3; ++v) {
-        const int cap = pair_cap_cols(4 >> v, R.max_rec);
         if (v > 0 && D.pr[v - 1].nitems && D.pr[v - 1].cols >= R.max_cols) { D.pr[v] = D.pr[v - 1]; continue; }
         PairItems O;
         // a proton core's rows all at once, or this many components are not taken together: every
         // part of its rows would gather all of x again
-        if (cap < R.max_cols || !build_pair_items(R, cap, O)) continue;
+        if (pair_cap_cols(4 >> v, R.max_rec) < R.max_cols || !build_pair_items(R, O)) continue;
         Device::PairDev &q = D.pr[v];
         if ((rc = put(D, q.items, O.items.data(), O.items.size(), err))) return rc;
         if ((rc = put(D, q.tiles, O.tiles.data(), O.tiles.size(), err))) return rc;
@@ -963,8 +962,7 @@ int bs_debug_table(bs_ctx *c, const char *name, void *out, int64_t *nbytes)
         else if (s.size() > 3 && s.substr(0, 3) == "pr_" && (s.back() == '1' || s.back() == '2' || s.back() == '4')) {
             // items for 1, 2 or 4 components at a time: "pr_items4", "pr_tiles4", "pr_rows4", "pr_store4", ...
             PairItems O;
-            const int cap = pair_cap_cols(s.back() - '0', T.pair.max_rec);
-            if (T.pair.on) build_pair_items(T.pair, cap, O);
+            if (T.pair.on && pair_cap_cols(s.back() - '0', T.pair.max_rec) >= T.pair.max_cols) build_pair_items(T.pair, O);
             auto raw = [&](const void *p, size_t b) {
                 tmp.assign((b + 7) / 8, 0);
                 if (b) std::memcpy(tmp.data(), p, b);

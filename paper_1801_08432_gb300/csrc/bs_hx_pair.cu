@@ -14,8 +14,8 @@
 // 0.84 and 1.03 ms at k = 4, 8, so k = 8 stays there.  The price is the multiply-adds with states the neutron core occupies
 // (their x is zero): ((ns - N + 1) / ns)^2 of them are of use, 0.72 at pf 4p4n.
 //
-// One CTA per SM and item: a proton core, or a range of its states when not
-// all rows fit, and CP of the K components.  The item's output rows Y live in
+// One CTA per SM and item: a proton core with all its rows and CP of the K
+// components.  The item's output rows Y live in
 // shared memory.  Four producer warps gather X (cp.async, zeros for occupied
 // states) and W into a ring of stages of KC pairs kl; sixteen consumer warps
 // in four groups share it: group g owns the rows of a fixed subset of the

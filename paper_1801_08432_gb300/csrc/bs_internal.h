@@ -534,7 +534,7 @@ void build_like_panels(const Basis &B, int spc, int pos, std::vector<LikePanel> 
 int like_panel_width(int max_n);
 bool like_applies(const bs_ctx *ctx);
 void build_pair_tables(const Basis &B, const Interaction &I, PairTables &T, int64_t max_cols);
-bool build_pair_items(const PairTables &T, int cap, PairItems &O);
+bool build_pair_items(const PairTables &T, PairItems &O);
 int pair_cap_cols(int cp, int max_rec);
 int upload(const Basis &B, const Interaction &I, const Tables &T, Device &D, std::string &err);
 void release(Device &D);

@@ -10,8 +10,9 @@
 // constant matrix W [pairs ij] x [pairs kl] takes to the elements of y.
 // Built here: the neutron cores grouped by (2M, parity) with the column of
 // every cn + s, the W matrix of every pair key (2m, parity), and per proton
-// core the list of its pairs, in items small enough for the output tile of
-// one CTA.
+// core the list of its pairs and, as the work of one CTA, its tiles.  Bases
+// whose proton cores have more output rows than the kernel's shared memory
+// holds have no items.
 #include <algorithm>
 #include <map>
 #include <new>
@@ -252,125 +253,101 @@ void build_pair_tables(const Basis &B, const Interaction &I, PairTables &T, int6
     T.on = !T.cores.empty();
 }
 
-// Items with at most cap output columns: a proton core and a range of its free states, largest work first.  False
-// where one state's rows alone exceed the cap.
-bool build_pair_items(const PairTables &T, int cap, PairItems &O)
+// Items, one for each proton core with all its free states, largest work first.  False where a core has more rows
+// than a tile can name.
+bool build_pair_items(const PairTables &T, PairItems &O)
 {
     O = PairItems();
     struct U { double cost; PairItem it; std::vector<PairTile> tiles; std::vector<PairRec> rows; std::vector<PairRow> store; };
     std::vector<U> units;
     for (const PairCore &pc : T.cores) {
-        // ranges of store rows (states in order) that fit; as even as the cap allows
-        const PairRow *rows = T.rows.data() + pc.row0;
-        int total = 0;
-        for (int r = 0; r < pc.nrow; ++r) total += rows[r].n;
-        const int nset = (total + cap - 1) / cap;
-        const int want = (total + nset - 1) / nset;
-        for (int r0 = 0; r0 < pc.nrow;) {
-            int r1 = r0, cols = 0;
-            while (r1 < pc.nrow) {   // whole states
-                int r2 = r1, c = 0;
-                while (r2 < pc.nrow && rows[r2].state == rows[r1].state) c += rows[r2++].n;
-                if (cols + c > cap) break;
-                if (cols && cols + c / 2 > want) break;
-                cols += c;
-                r1 = r2;
-            }
-            if (r1 == r0) return false;
-            U u;
-            const int ybase = rows[r0].ycol;
-            u.it.rec0 = pc.rec0;
-            u.it.nrec = pc.nrec;
-            u.it.cols = cols;
-            for (int r = r0; r < r1; ++r) {
-                u.store.push_back(rows[r]);
-                u.store.back().ycol -= ybase;
-            }
-            // the states in four subsets, one per consumer group: each state, the one
-            // with the most rows first, to the subset whose fullest neutron group grows least
-            std::vector<int> states;
-            for (int r = r0; r < r1; ++r)
-                if (states.empty() || states.back() != rows[r].state) states.push_back(rows[r].state);
-            std::vector<std::vector<int>> cnt(states.size(), std::vector<int>((size_t)pc.ngrp, 0));
-            std::vector<int> sub(64, -1);
-            std::vector<size_t> by(states.size());
-            std::vector<long> tot(states.size(), 0);
-            for (size_t a = 0; a < states.size(); ++a) {
-                by[a] = a;
-                for (int g = 0; g < pc.ngrp; ++g) {
-                    const PairGroup &G = T.grps[(size_t)(pc.grp0 + g)];
-                    const uint8_t *st = T.rec_state.data() + pc.rec0 + G.rec0;
-                    for (int r = 0; r < G.nrec; ++r) cnt[a][(size_t)g] += st[r] == states[a];
-                    tot[a] += (long)cnt[a][(size_t)g] * G.nrec;
-                }
-            }
-            std::stable_sort(by.begin(), by.end(), [&](size_t a, size_t b) { return tot[a] > tot[b]; });
-            std::vector<std::vector<int>> load(4, std::vector<int>((size_t)pc.ngrp, 0));
-            for (size_t a : by) {
-                int best = 0;
-                double bestc = 1e300;
-                for (int q = 0; q < 4; ++q) {
-                    double c = 0;   // sum over groups of (load after)^2, heavier for long sums
-                    for (int g = 0; g < pc.ngrp; ++g) {
-                        const double l = load[(size_t)q][(size_t)g], n = cnt[a][(size_t)g];
-                        c += ((l + n) * (l + n) - l * l) * T.grps[(size_t)(pc.grp0 + g)].nrec;
-                    }
-                    if (c < bestc) { bestc = c; best = q; }
-                }
-                sub[(size_t)states[a]] = best;
-                for (int g = 0; g < pc.ngrp; ++g) load[(size_t)best][(size_t)g] += cnt[a][(size_t)g];
-            }
-            u.cost = 2.0 * cols;
+        U u;
+        u.it = {};
+        u.it.rec0 = pc.rec0;
+        u.it.nrec = pc.nrec;
+        u.store.assign(T.rows.begin() + pc.row0, T.rows.begin() + pc.row0 + pc.nrow);
+        for (const PairRow &r : u.store) u.it.cols += r.n;
+        // the states in four subsets, one per consumer group: each state, the one
+        // with the most rows first, to the subset whose fullest neutron group grows least
+        std::vector<int> states;
+        for (const PairRow &r : u.store)
+            if (states.empty() || states.back() != r.state) states.push_back(r.state);
+        std::vector<std::vector<int>> cnt(states.size(), std::vector<int>((size_t)pc.ngrp, 0));
+        std::vector<int> sub(64, -1);
+        std::vector<size_t> by(states.size());
+        std::vector<long> tot(states.size(), 0);
+        for (size_t a = 0; a < states.size(); ++a) {
+            by[a] = a;
             for (int g = 0; g < pc.ngrp; ++g) {
                 const PairGroup &G = T.grps[(size_t)(pc.grp0 + g)];
-                std::vector<PairRec> list[4];
-                for (int r = 0; r < G.nrec; ++r) {
-                    const int q = sub[T.rec_state[(size_t)(pc.rec0 + G.rec0 + r)]];
-                    if (q < 0) continue;
-                    list[q].push_back(T.recs[(size_t)(pc.rec0 + G.rec0 + r)]);
-                    list[q].back().yoff -= (uint32_t)ybase;
+                const uint8_t *st = T.rec_state.data() + pc.rec0 + G.rec0;
+                for (int r = 0; r < G.nrec; ++r) cnt[a][(size_t)g] += st[r] == states[a];
+                tot[a] += (long)cnt[a][(size_t)g] * G.nrec;
+            }
+        }
+        std::stable_sort(by.begin(), by.end(), [&](size_t a, size_t b) { return tot[a] > tot[b]; });
+        std::vector<std::vector<int>> load(4, std::vector<int>((size_t)pc.ngrp, 0));
+        for (size_t a : by) {
+            int best = 0;
+            double bestc = 1e300;
+            for (int q = 0; q < 4; ++q) {
+                double c = 0;   // sum over groups of (load after)^2, heavier for long sums
+                for (int g = 0; g < pc.ngrp; ++g) {
+                    const double l = load[(size_t)q][(size_t)g], n = cnt[a][(size_t)g];
+                    c += ((l + n) * (l + n) - l * l) * T.grps[(size_t)(pc.grp0 + g)].nrec;
                 }
-                size_t most = 0;
-                for (auto &v : list) {
-                    std::stable_sort(v.begin(), v.end(), [](const PairRec &a, const PairRec &b) { return a.wj >> 24 < b.wj >> 24; });
-                    most = std::max(most, v.size());
+                if (c < bestc) { bestc = c; best = q; }
+            }
+            sub[(size_t)states[a]] = best;
+            for (int g = 0; g < pc.ngrp; ++g) load[(size_t)best][(size_t)g] += cnt[a][(size_t)g];
+        }
+        u.cost = 2.0 * u.it.cols;
+        for (int g = 0; g < pc.ngrp; ++g) {
+            const PairGroup &G = T.grps[(size_t)(pc.grp0 + g)];
+            std::vector<PairRec> list[4];
+            for (int r = 0; r < G.nrec; ++r) {
+                const int q = sub[T.rec_state[(size_t)(pc.rec0 + G.rec0 + r)]];
+                list[q].push_back(T.recs[(size_t)(pc.rec0 + G.rec0 + r)]);
+            }
+            size_t most = 0;
+            for (auto &v : list) {
+                std::stable_sort(v.begin(), v.end(), [](const PairRec &a, const PairRec &b) { return a.wj >> 24 < b.wj >> 24; });
+                most = std::max(most, v.size());
+            }
+            const int nch = (G.ncore + kPairCores - 1) / kPairCores;
+            const int ch = ((G.ncore + nch - 1) / nch + 31) / 32 * 32;
+            for (size_t p0 = 0; p0 < most; p0 += kPairRows) {
+                PairTile t = {};
+                t.rec0 = G.rec0;
+                t.nrec = G.nrec;
+                t.woff = G.woff;
+                t.np = G.np;
+                int rmax = 0;
+                for (int q = 0; q < 4; ++q) {
+                    t.row0[q] = (uint16_t)u.rows.size();
+                    const size_t n = list[q].size() > p0 ? std::min<size_t>(kPairRows, list[q].size() - p0) : 0;
+                    t.nrow[q] = (uint8_t)n;
+                    rmax = std::max(rmax, (int)n);
+                    t.first[q] = n > 0;
+                    for (size_t r = 0; r < n; ++r) {
+                        if (r && list[q][p0 + r].wj >> 24 != list[q][p0 + r - 1].wj >> 24) t.first[q] |= (uint16_t)(1u << r);
+                        u.rows.push_back(list[q][p0 + r]);
+                    }
                 }
-                const int nch = (G.ncore + kPairCores - 1) / kPairCores;
-                const int ch = ((G.ncore + nch - 1) / nch + 31) / 32 * 32;
-                for (size_t p0 = 0; p0 < most; p0 += kPairRows) {
-                    PairTile t = {};
-                    t.rec0 = G.rec0;
-                    t.nrec = G.nrec;
-                    t.woff = G.woff;
-                    t.np = G.np;
-                    int rmax = 0;
-                    for (int q = 0; q < 4; ++q) {
-                        t.row0[q] = (uint16_t)u.rows.size();
-                        const size_t n = list[q].size() > p0 ? std::min<size_t>(kPairRows, list[q].size() - p0) : 0;
-                        t.nrow[q] = (uint8_t)n;
-                        rmax = std::max(rmax, (int)n);
-                        t.first[q] = n > 0;
-                        for (size_t r = 0; r < n; ++r) {
-                            if (r && list[q][p0 + r].wj >> 24 != list[q][p0 + r - 1].wj >> 24) t.first[q] |= (uint16_t)(1u << r);
-                            u.rows.push_back(list[q][p0 + r]);
-                        }
-                    }
-                    for (int c0 = 0; c0 < G.ncore; c0 += ch) {
-                        t.core0 = G.core0 + c0;
-                        t.ncore = std::min(ch, G.ncore - c0);
-                        u.tiles.push_back(t);
-                        u.cost += (double)G.nrec * (rmax + 3) * (0.5 + t.ncore / 256.0) + 100.0;
-                    }
+                for (int c0 = 0; c0 < G.ncore; c0 += ch) {
+                    t.core0 = G.core0 + c0;
+                    t.ncore = std::min(ch, G.ncore - c0);
+                    u.tiles.push_back(t);
+                    u.cost += (double)G.nrec * (rmax + 3) * (0.5 + t.ncore / 256.0) + 100.0;
                 }
             }
-            if (u.rows.size() > 65535) return false;
-            O.max_cols = std::max(O.max_cols, cols);
-            O.max_tiles = std::max(O.max_tiles, (int)u.tiles.size());
-            O.max_rows = std::max(O.max_rows, (int)u.rows.size());
-            O.max_rec = std::max(O.max_rec, pc.nrec);
-            units.push_back(std::move(u));
-            r0 = r1;
         }
+        if (u.rows.size() > 65535) return false;
+        O.max_cols = std::max(O.max_cols, u.it.cols);
+        O.max_tiles = std::max(O.max_tiles, (int)u.tiles.size());
+        O.max_rows = std::max(O.max_rows, (int)u.rows.size());
+        O.max_rec = std::max(O.max_rec, pc.nrec);
+        units.push_back(std::move(u));
     }
     std::stable_sort(units.begin(), units.end(), [](const U &a, const U &b) { return a.cost > b.cost; });
     for (U &u : units) {
