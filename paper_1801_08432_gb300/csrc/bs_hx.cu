@@ -283,26 +283,41 @@ int launch_hx(const bs_ctx *c, const void *x, void *y, int k, bs_dtype dt, void 
     if (mode == 0) mode = c->tuned[dt == BS_F64 ? 0 : 1][kslot(k)];
     if (mode == 0 && e == cudaSuccess) {
         const int64_t dim = c->basis.dim;
+        // Columns of the widest neutron sector, proton rows (the CTAs of the row and pipelined kernels), and CTAs
+        // that fill the chip (one per SM).
+        const int nN = c->dev.max_nN, rows = c->dev.nrtasks, chip = c->tab.grid;
         if (dt == BS_F64 || c->dev.trunc) {
-            // the first pipelined variant, else the first row variant, else the tiled kernel; small bases the tiled
-            // kernel (FP64 k = 1, us, tiled / row: sd 2p2n 15 / 37, sd 4p4n 70 / 95, pf 2p3n 62 / 68, sd 5p6n 182 / 133)
-            if (dim < 50000) {
+            // The first pipelined variant, else the first row variant, else the tiled kernel; small bases the tiled
+            // kernel, but where the pipelined one (k >= 2) has a full chip of rows and wide sectors to work on.
+            // FP64, us, tiled / row / pipelined at k = 1, 2, 4, 8:
+            //   sd 2p2n 9 / 37 / -, 11 / 39 / 28, 15 / 51 / 37, 21 / 71 / 60;  sd 4p4n (495 rows, 81 columns) 64 / 95 / -,
+            //   93 / 117 / 126, 152 / 178 / 150, 244 / 561 / 334;  sd 3p5n (220, 119) 50 / 53 / -, 74 / 66 / 64,
+            //   115 / 101 / 88, 201 / 286 / 172;  pf 2p3n (190, 145) 60 / 68 / -, 89 / 85 / 75, 131 / 132 / 113, 254 / 340 / 222;
+            //   sd 5p5n (69,784 states) 146 / 127 / -, 223 / 213 / 230, 375 / 341 / 308, 620 / 1047 / 597.
+            if (dim < 50000 && !(k > 1 && rows >= chip && nN >= 96)) {
                 mode = 1;
             } else {
                 e = launch_hx_pipe(c, x, y, k, dt, s, 0, used);
                 if (!used) mode = 2;
             }
         } else {
-            // FP32, not tuned.  Measured on this chip, us per product of k = 4 (k = 2) by the tiled / pipelined
-            // (row) / core-grouped / pair-core kernels:
-            //   sd 4p4n 34 / 51 / 82 / 67 (31 / 71 / - / 56);  pf 3p3n 126 / 152 / 168 / 163 (100 / 179 / - / 109);
-            //   pf 4p3n 512 / 741 / 929 / 685 (400 / 762 / - / 353);  pf 4p4n 2761 / 2103 / 1232 / 1141 (1820 / 2236 / - / 725);
-            //   pf 6p2n (neutron sectors of 30) 892 / 5779 / 9782 / - (743 / 4947 / - / -);
-            // at k = 8 the core-grouped kernels lead from 100,000 states and sectors of 64 columns on.
-            const int nN = c->dev.max_nN;
-            if (dim < 100000 || nN < 64) mode = 1;                     // (the wide kernels give a thread a column)
-            else if (k < 4) mode = kPairMode;
-            else if (k == 4) mode = nN < 256 ? 1 : kPairMode;
+            // FP32, not tuned; us per product by the tiled / row / pair-core kernels at k = 1 and 2:
+            //   sd 4p4n 21 / 69 / 52, 25 / 71 / 54;  pf 2p4n (190 rows, 565 columns) 72 / 91 / 109, 87 / 106 / 121;
+            //   pf 3p3n 94 / 170 / 101, 111 / 179 / 107;  pf 2p5n (20 proton cores) 237 / 213 / 268, 339 / 290 / -;
+            //   pf 4p3n 384 / 714 / 316, 398 / 761 / 353;  pf 4p4n 1835 / 1779 / 580, 2096 / 2232 / 721;
+            //   pf 6p2n (sectors of 30 columns) 736 / 4956 / -, 724 / 4975 / -;
+            // by the tiled / pipelined / core-grouped (20) / pair-core kernels at k = 4 and 8:
+            //   sd 4p4n 27 / 50 / 83 / 67, 39 / 72 / 86 / 89;  pf 2p4n 111 / 97 / 70 / 166, 185 / 177 / 91 / 180;
+            //   pf 3p3n 127 / 152 / 167 / 162, 210 / 238 / 185 / 228;  pf 4p3n 500 / 741 / 929 / 689, 943 / 1166 / 1001 / 1084;
+            //   pf 3p4n (190 proton cores) 648 / 437 / 239 / 276, 1188 / 788 / 330 / 451;
+            //   pf 4p4n (1,140) 2781 / 2107 / 1231 / 1140, 5454 / 3915 / 1582 / 2008;  pf 6p2n 888 / 5798 / 9786 / 6620.
+            // So: the tiled kernel for narrow sectors (the wide kernels give a thread a column) and small bases, but from
+            // k = 4 on not where a full chip of rows is 256 columns wide; pairs of cores (a CTA each) where the proton
+            // cores fill the chip, at k = 4 three times; the core-grouped kernel else.
+            const int cores = c->dev.pr[k == 1 ? 2 : k == 2 ? 1 : 0].nitems;
+            if (nN < 64 || (dim < 100000 && (k < 4 || nN < 256 || rows < chip))) mode = 1;
+            else if (k < 4) mode = cores >= chip ? kPairMode : 2;
+            else if (k == 4) mode = nN < 256 ? 1 : cores >= 3 * chip ? kPairMode : kCoreMode;
             else mode = kCoreMode;
             if (mode == kPairMode || mode == kCoreMode) {
                 // a form that does not fit this basis: the next one
