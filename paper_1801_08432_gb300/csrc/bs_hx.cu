@@ -233,13 +233,14 @@ cudaError_t launch(const Device &Dv, const DevCoefs<T> &C, const T *x, T *y, cud
         hx_fused_kernel<T, K, NT><<<Dv.ntasks, NT, 0, s>>>(A, C.pp_coef, C.nn_coef, C.wpn, C.ppx_coef, C.nnx_coef, x, y);
     };
     // Threads by the number of CTAs: with few, more groups shorten each thread's chain of loads; with many, they only
-    // take registers.  us at 128 / 256 / 512 threads (with the pn links walked one by one; the flat jump lists take
-    // a third off the small ones): sd 2p2n (66 CTAs) FP64 k = 1 17 / 15 / 16; sd 4p4n (495) FP32
-    // k = 4 51 / 37 / 34, k = 8 64 / 47 / 49, FP64 k = 8 297 / 254 / 293; pf 3p3n (2,200) k = 1 111 / 98 / 130,
-    // k = 4 126 / 154 / 152, k = 8 228 / 219 / 249; pf 4p3n (9,500) k = 1 398 / 413 / 585.
+    // take registers.  us at 128 / 256 / 512 threads: sd 2p2n (66 CTAs) FP64 k = 1 15 / 11 / 9; sd 4p4n (495) FP32
+    // k = 1 46 / 29 / 21, k = 4 52 / 31 / 27, k = 8 62 / 43 / 39, FP64 k = 4 183 / 148 / 152, k = 8 298 / 245 / -;
+    // pf 3p3n (2,200) FP32 k = 1 110 / 95 / 92, k = 2 111 / 105 / 106, k = 4 128 / 124 / 130, k = 8 218 / 211 / 209, FP64
+    // k = 1 383 / 332 / 321, k = 4 938 / 824 / 857; pf 4p3n (7,000) FP32 k = 1 384 / 382 / 402, k = 2 398 / 416 / 474,
+    // k = 4 501 / 549 / 592; pf 6p2n (35,000) FP32 k = 1 734 / 827 / 995, k = 4 896 / 1210 / 1455.
     constexpr bool wide = K * sizeof(T) == 64;
     if (Dv.ntasks < 1000 && !wide) run(std::integral_constant<int, 512>{});
-    else if (Dv.ntasks < 1000 || (Dv.ntasks < 2500 && (K == 1 || K == 8))) run(std::integral_constant<int, 256>{});
+    else if (Dv.ntasks < 2500) run(std::integral_constant<int, 256>{});
     else run(std::integral_constant<int, 128>{});
     return cudaGetLastError();
 }
