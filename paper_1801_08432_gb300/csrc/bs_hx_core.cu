@@ -1101,9 +1101,11 @@ cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dt
         e = k == 8 ? launch_nn_k<8>(c, nullptr, nullptr, s, R, fits) : launch_nn_k<4>(c, nullptr, nullptr, s, R, fits);
     } else {
         // nn by tiles of three or two rows into one more partial vector where they fit (a list entry is read once for
-        // all of them: pf 6p6n k = 4, 17 ms by the row at a time, 14.4 by two, 13.1 by three), else by the first
+        // all of them: pf 6p6n k = 4, 17 ms by the row at a time, 14.4 by two, 13.1 by three) and give every SM a
+        // tile (pf 1p5n k = 8, four rows a sector: the product 237 us by tiles, 176 by the row), else by the first
         // pipelined variant that fits
         for (int r = 3; pp && !nrow && r >= 2 && e == cudaSuccess; --r) {
+            if ((r == 3 ? c->dev.nnntasks3 : c->dev.nnntasks2) < c->tab.grid) continue;
             e = k == 8 ? launch_nn_k<8>(c, nullptr, nullptr, s, r, fits) : launch_nn_k<4>(c, nullptr, nullptr, s, r, fits);
             if (fits) nrow = r;
         }
