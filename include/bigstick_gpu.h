@@ -151,8 +151,8 @@ int bs_load_interaction(bs_ctx *ctx, const double *spe, int n_spe,
  * x, y: device, [dim][k], dtype elements, distinct (no aliasing).  BS_F64
  * computes in double; BS_F32 reads/writes float and accumulates in float
  * with coefficients rounded once from the FP64 decoupling.  y is fully
- * overwritten.  Deterministic: every element of y is owned by one thread and
- * summed in a fixed order.  Errors: BS_ENOBASIS, BS_ENOINT, BS_EINVAL, BS_ECUDA. */
+ * overwritten.  Deterministic: every element of y is summed in a fixed order
+ * (one that depends on the kernel mode).  Errors: BS_ENOBASIS, BS_ENOINT, BS_EINVAL, BS_ECUDA. */
 int bs_apply_H(bs_ctx *ctx, const void *x, void *y, int k, bs_dtype dtype, void *stream);
 
 /* The same product with HOST buffers x_host, y_host ([dim][k]); copies in,
@@ -417,13 +417,14 @@ int bs_debug_eigh_banded(int n, int bw, const double *A, int nval, double *w, do
  * neutron-list buffers; 17, 18, 19: 227 KB, two list buffers; 20: 227 KB,
  * three list buffers; 16: the pn term by pairs of a (Z-1)-proton and an
  * (N-1)-neutron core, a dense product per group of neutron cores, for every
- * k); in 11, 12, 17
+ * k -- recorded tunings from before that kernel mean by 16 the variant of 15
+ * with four list buffers, which is gone); in 11, 12, 17
  * the pipelined kernel computes the like-particle terms into one more (17:
  * the first pipelined variant that fits, for neutron sectors wider than 576
  * columns); in 13..16 and 18..20 a second persistent kernel computes the pp
  * two-body term per
  * (Z-2)-proton core into C(Z,2) more and a row-tile kernel (4 rows per CTA,
- * 2 in 19 and 20, column tiles of 576 for wider sectors; 18: 3 or 2, whichever
+ * 2 in 16, 19 and 20, column tiles of 576 for wider sectors; 18: 3 or 2, whichever
  * fits first, into one more partial vector, else the first pipelined variant
  * that fits) the nn term and the proton single-particle energies
  * into one more (16 with k = 1, 2: panels of x in shared memory for

@@ -886,15 +886,15 @@ struct CoreVariant {
     bool pair;       // the pn term by pairs of cores (bs_hx_pair.cu) instead
 };
 
-// Modes 11.. in this order.  The last two spend the whole 227 KB on three or
-// four list buffers: the producer can then run two or three link groups
-// ahead of the slowest consumer warp instead of one.
-// Modes 17, 18 also spend 227 KB, with two list buffers, and leave the
-// like-particle terms (17: pp and nn; 18: nn, after the pp-core kernel) to
-// the first pipelined variant that fits the basis: for source rows of up to
-// ~64 KB (pf 6p6n: 3,952 columns of 16 bytes at k = 4).  Mode 19 is 18 with
-// the nn term in row tiles of 2 rows (two CTAs per SM); mode 20 pairs those
-// 2-row tiles with the three list buffers of mode 15.
+// Modes 11.. in this order.  Mode 15 spends the whole 227 KB on three list
+// buffers: the producer can then run two link groups ahead of the slowest
+// consumer warp instead of one.  Mode 16 forms the pn term by pairs of cores.
+// Modes 17, 18 also spend 227 KB, with two list buffers, for source rows of
+// up to ~64 KB (pf 6p6n: 3,952 columns of 16 bytes at k = 4); 17 leaves the
+// like-particle terms to the first pipelined variant that fits the basis, 18
+// takes pp by cores and nn in tiles of three or two rows where they fit.
+// Mode 19 is 18 with the nn term and the ordered sum in tiles of 2 rows (two
+// CTAs per SM); mode 20 pairs those with the three list buffers of mode 15.
 constexpr CoreVariant kCoreVariants[] = {{18, 1, 200 * 1024, false, 0, 0}, {9, 2, 200 * 1024, false, 0, 0},
                                          {18, 1, 200 * 1024, true, 4, 0},  {9, 2, 200 * 1024, true, 4, 0},
                                          {18, 1, 227 * 1024, true, 4, 3},  {18, 1, 227 * 1024, true, 2, 2, true},
@@ -1061,9 +1061,9 @@ void release_hx_old(const bs_ctx *c)
     c->core_part_captured = false;
 }
 
-// Core-grouped pn kernel variant v followed by the pipelined like-particle
-// kernel (variant 0) that adds the partials; `used` is false when the path
-// does not apply (FP64, k < 4, no cores) or does not fit.
+// pn kernel of variant v (k = 1, 2: by pairs of cores only), then the
+// like-particle terms and the ordered sum of the partial vectors; `used` is
+// false when the path does not apply (FP64, no cores) or does not fit.
 cudaError_t launch_hx_core(const bs_ctx *c, const void *x, void *y, int k, bs_dtype dt, cudaStream_t s, int v,
                            bool &used, cudaEvent_t t0, cudaEvent_t t1)
 {

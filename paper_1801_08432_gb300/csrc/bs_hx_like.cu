@@ -70,7 +70,6 @@ struct LikeArgs {
     const float *part;     // pp: partial vectors to add, nz of them
     int nz;
     int64_t pstride;
-    int max_n;
 };
 
 // PW floats of a panel row (64 or 32); NN: the acting species is the neutrons.
@@ -200,7 +199,7 @@ cudaError_t launch_like_t(int dev, const Device::LikeDev &L, const float *x, flo
     auto kern = hx_like_kernel<K, PW, NN>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    LikeArgs A{L.panels[K - 1], L.ptr, L.ent, part, nz, pstride, L.max_n};
+    LikeArgs A{L.panels[K - 1], L.ptr, L.ent, part, nz, pstride};
     const int np = L.npanels[K - 1];
     if (np <= 0) return cudaSuccess;
     // several CTAs to a panel, each with some of its rows, until there are four for every

@@ -538,14 +538,14 @@ struct LState {
 // once per group of blocks.  Consumer thread (r, j), r < 256 / K, owns
 // column j of the rows r + (256 / K) m, m < kRsRT, of each tile.
 //
-// Dot products: each thread sums its kRsRT rows (FP32 FMAs unless EXACT),
+// Dot products (rs_dots): each thread sums its kRsRT rows (FP32 or FP64 FMAs),
 // the lanes of a warp with equal j are combined (the first two steps in
 // FP32, so a plain FP32 sum never spans more than 4 kRsRT = 32 products;
 // then double-float), the 8 warps in a fixed order, and the tile's K x K
 // result is added to the CTA's double-float partial in global memory, which
 // dots_reduce sums over CTAs in FP64 in a fixed order: deterministic.
-// EXACT forms every product exactly (p + fma residual) in double-float, as
-// the row-slot kernel does.  FP64 vectors use FP64 throughout.
+// FP64 vectors use FP64 throughout.  Exact products of FP32 vectors are
+// formed by rs_dots_x, below.
 // The update applies, per output element, the blocks in order and within a
 // block i = 0..K-1, the order of blk_update, so both give identical W.
 // Applicability: 16-byte aligned V, W and block stride (the TMA rule) and
@@ -656,13 +656,13 @@ constexpr int kRsSR = 4;   // staging slots of warp results
 constexpr int kRsLaneIS = 36;
 constexpr int kRsLaneSR = 2;
 
-template <typename T, int K, bool EXACT>
+template <typename T, int K>
 __host__ __device__ constexpr bool rs_lane_staging()
 {
-    return std::is_same<T, float>::value && !EXACT && K == 8;
+    return std::is_same<T, float>::value && K == 8;
 }
 
-template <typename T, int K, bool EXACT, int S>
+template <typename T, int K, int S>
 __global__ void __launch_bounds__(kRsCons + 64, sizeof(T) == 4 ? 2 : 1)
     rs_dots(const T *__restrict__ V, int64_t bstride, int nb, const T *__restrict__ W, int64_t nel,
             typename RsRed<T>::S *__restrict__ partial, int acc_in_smem, const int *__restrict__ nb_iter, int *err)
@@ -672,8 +672,8 @@ __global__ void __launch_bounds__(kRsCons + 64, sizeof(T) == 4 ? 2 : 1)
     using Sv = typename R::S;
     constexpr int NR = kRsCons / K;
     constexpr int NCW = kRsCons / 32;   // consumer warps
-    constexpr bool PACKED = std::is_same<T, float>::value && !EXACT && K >= 2;   // two-wide FP32 FMAs
-    constexpr bool LANES = rs_lane_staging<T, K, EXACT>();
+    constexpr bool PACKED = std::is_same<T, float>::value && K >= 2;   // two-wide FP32 FMAs
+    constexpr bool LANES = rs_lane_staging<T, K>();
     constexpr int SR = LANES ? kRsLaneSR : kRsSR;
     constexpr int SLOT = LANES ? NCW * K * kRsLaneIS * 4 : NCW * K * K * (int)sizeof(Sv);   // bytes per staging slot
     if (nb_iter) nb = *nb_iter + 1;   // graph replay: blocks 0..n of iteration n
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(kRsCons + 64, sizeof(T) == 4 ? 2 : 1)
                 for (int o = 4 * K; o < 32; o <<= 1)
 #pragma unroll
                     for (int j = 0; j < K; ++j) sum[j] = R::add(sum[j], R::shfl(sum[j], o));
-            } else if constexpr (std::is_same<T, float>::value && !EXACT) {   // K = 1
+            } else if constexpr (std::is_same<T, float>::value) {   // K = 1
                 float acc = 0.f;
                 if (!bad) {
 #pragma unroll
@@ -1504,7 +1504,7 @@ void dots(LState &L, const T *V, int nb, const T *W, double *out, const int *nb_
         using Sv = typename RsRed<T>::S;
         constexpr int S = rs_stages<T>();
         const size_t acc = (size_t)(nb_iter ? nb_max : nb) * K * K * sizeof(Sv);
-        constexpr bool LANES = rs_lane_staging<T, K, EXACT>();
+        constexpr bool LANES = rs_lane_staging<T, K>();
         const size_t slots = LANES ? (size_t)kRsLaneSR * 8 * K * kRsLaneIS * 4 : (size_t)kRsSR * 8 * K * K * sizeof(Sv);
         const size_t fixed = 256 + (size_t)S * kRsCE * sizeof(T) + slots;
         const int acc_in_smem = fixed + acc <= 113 * 1024;
@@ -1513,10 +1513,10 @@ void dots(LState &L, const T *V, int nb, const T *W, double *out, const int *nb_
         int dev = 0;
         cudaGetDevice(&dev);
         if (dev < 64 && !(attr >> dev & 1ull)) {
-            cudaFuncSetAttribute(rs_dots<T, K, EXACT, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
+            cudaFuncSetAttribute(rs_dots<T, K, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
             attr |= 1ull << dev;
         }
-        rs_dots<T, K, EXACT, S><<<L.ncta, kRsCons + 64, smem, L.s>>>(V, L.bstride, nb, W, L.dim * K,
+        rs_dots<T, K, S><<<L.ncta, kRsCons + 64, smem, L.s>>>(V, L.bstride, nb, W, L.dim * K,
                                                                      reinterpret_cast<Sv *>(L.partial), acc_in_smem,
                                                                      nb_iter, L.err);
         reduce_parts<Sv>(reinterpret_cast<const Sv *>(L.partial), L.ncta, n, nb * K * K, out, nb_iter, out_iter, K * K,
