@@ -1550,9 +1550,14 @@ void update(LState &L, const T *V, int nb, const double *C, T *W, const int *nb_
     constexpr int S = sizeof(T) == 4 ? 3 : 2;   // 16 KB (FP32) or 32 KB (FP64) tiles
     const size_t rsm = 128 + (size_t)S * kRsCEU * sizeof(T) + csm;
     if (rs_applies<T, K>(L, V, W) && rsm <= 112 * 1024) {
-        // tiles of one row per thread where the larger ones (more rows per read of C) leave CTAs without any:
-        // sd 4p4n k = 4, 28 tiles for 304 CTAs, 9.9 -> 8.7 us a pass
-        if (L.dim * K < (int64_t)kRsCEU * L.ncta) launch_update<T, K, S, kRsCons * K>(L, V, nb, C, W, nb_iter, c_iter, csm);
+        // Tiles of one row per thread where the larger ones (more rows per read of C) leave CTAs without any.  FP32: while
+        // a CTA has one such tile, at k = 8 an SM; us, large / one-row tiles, 24 blocks: sd 4p4n k = 4 (112 one-row tiles)
+        // 10.4 / 10.3 (40 blocks 16.5 / 12.4), sd 5p5n (273) k = 1 10.3 / 8.3, sd 4p5n (173) k = 8 15.3 / 18.5, sd 6p6n (367)
+        // k = 4 10.7 / 14.5, pf 5p2n (1,025) k = 4 18 / 33.  FP64: wherever large ones are fewer than the CTAs: sd 4p4n
+        // k = 2 55 / 12, pf 3p3n k = 4 197 / 102, k = 8 (238 large ones) 392 / 390.
+        const int64_t tiles = (L.dim + kRsCons - 1) / kRsCons;
+        if (sizeof(T) == 8 ? L.dim * K < (int64_t)kRsCEU * L.ncta : tiles <= (K == 8 ? L.ncta / 2 : L.ncta))
+            launch_update<T, K, S, kRsCons * K>(L, V, nb, C, W, nb_iter, c_iter, csm);
         else launch_update<T, K, S, kRsCEU>(L, V, nb, C, W, nb_iter, c_iter, csm);
         return;
     }
