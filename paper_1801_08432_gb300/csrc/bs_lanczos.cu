@@ -1588,9 +1588,14 @@ static int lanczos_run(bs_ctx *c, const bs_lanczos_opts &o, const void *pivot, d
     niter = (int)std::min<int64_t>(niter, std::max<int64_t>(1, L.dim / K));
     const size_t es = sizeof(T);
     std::vector<void *> owned;
+    bool short_of = false;   // an allocation failed
     auto alloc = [&](size_t bytes) -> void * {
         void *p = nullptr;
-        if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) return nullptr;
+        if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            short_of = true;
+            return nullptr;
+        }
         owned.push_back(p);
         return p;
     };
@@ -1629,8 +1634,7 @@ static int lanczos_run(bs_ctx *c, const bs_lanczos_opts &o, const void *pivot, d
     L.Ahist = (double *)alloc((size_t)niter * K * K * sizeof(double));
     L.Bhist = (double *)alloc((size_t)niter * K * K * sizeof(double));
     L.flags = (int *)alloc(sizeof(int));
-    for (void *p : owned)
-        if (!p) { cleanup(); c->err = "lanczos: device allocation failed"; return BS_ENOMEM; }
+    if (short_of) { cleanup(); c->err = "lanczos: device allocation failed"; return BS_ENOMEM; }
     {
         cudaError_t e = cudaFuncSetAttribute(blk_update<T, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)std::min<size_t>((size_t)(niter + 1) * K * K * es, 227 * 1024));
