@@ -1061,6 +1061,17 @@ void release_hx_old(const bs_ctx *c)
     c->core_part_captured = false;
 }
 
+// Gives the workspace up (products that use it then run by other kernels where it cannot be had again); false where there
+// is none, or a graph may hold it.
+bool drop_hx_part(const bs_ctx *c)
+{
+    if (!c->core_part || c->core_part_captured) return false;
+    cudaFree(c->core_part);
+    c->core_part = nullptr;
+    c->core_part_bytes = 0;
+    return true;
+}
+
 // pn kernel of variant v (k = 1, 2: by pairs of cores only), then the
 // like-particle terms and the ordered sum of the partial vectors; `used` is
 // false when the path does not apply (FP64, no cores) or does not fit.

@@ -562,4 +562,5 @@ int core_variants();
 // allocates what launch_hx needs for (k, dtype) outside any stream capture
 int prepare_hx(const bs_ctx *ctx, int k, bs_dtype dt, std::string &err);
 void release_hx_old(const bs_ctx *ctx);
+bool drop_hx_part(const bs_ctx *ctx);
 }  // namespace bs

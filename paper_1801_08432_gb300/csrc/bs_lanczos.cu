@@ -1591,7 +1591,12 @@ static int lanczos_run(bs_ctx *c, const bs_lanczos_opts &o, const void *pivot, d
     bool short_of = false;   // an allocation failed
     auto alloc = [&](size_t bytes) -> void * {
         void *p = nullptr;
-        if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) {
+        cudaError_t e = cudaMalloc(&p, std::max<size_t>(bytes, 16));
+        if (e == cudaErrorMemoryAllocation && drop_hx_part(c)) {   // the stored basis before the products' workspace
+            (void)cudaGetLastError();
+            e = cudaMalloc(&p, std::max<size_t>(bytes, 16));
+        }
+        if (e != cudaSuccess) {
             (void)cudaGetLastError();
             short_of = true;
             return nullptr;
