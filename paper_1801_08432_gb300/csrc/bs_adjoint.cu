@@ -348,7 +348,7 @@ __device__ __forceinline__ void gput(T *p, const T (&v)[K])
 // operations bound it (K multiply-adds and 7 adds per pair and column) or
 // FP64 ones.  48Cr k = 4: 26.7 ms for pn alone with an FP64 shared-memory
 // atomic per pair of jumps, 2.3 ms with every pair of the key in fixed
-// threads, 2.0 ms this way (a third of the FP32 pipe; many small units).
+// threads, 2.1 ms this way (0.44 of the FP32 pipe; many small units).
 template <typename T>
 __host__ __device__ constexpr int gram_lg(int e) { return e == 4 ? 6 : e == 8 ? 5 : e == 16 ? 4 : e == 32 ? 3 : 2; }   // 2^lg columns of 128 pairs fit
 template <typename T, int K>

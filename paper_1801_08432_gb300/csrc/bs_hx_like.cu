@@ -10,7 +10,8 @@
 // its 32 lanes hold the row's columns, so the list entry (source, coefficient)
 // is the same for all lanes and the source row is read without bank
 // conflicts, 2 wavefronts per 64 multiply-adds.  Shared-memory wavefronts
-// bound it (2.5 per entry, 0.5 of them the entry's own broadcast read).
+// bound it (3.3 per entry at pf 4p4n k = 2: 0.5 the entry's own broadcast
+// read, 0.8 the staging; L1 85 % busy in the nn kernel).
 // Against lists per lane (a lane gathers its own column's sources) this reads
 // no padding and no conflicts, and an entry costs 8 bytes per 64
 // multiply-adds instead of 8 bytes per lane: 0.19 ms for both terms at pf

@@ -6,17 +6,17 @@
 // (Z-1)-core kernel, which gathers an element of x once per neutron jump for
 // at most four rows, an element is gathered once per (proton, neutron)
 // particle pair it holds and feeds every pair ij: 14 times fewer gathers at
-// pf 4p4n.  What bounds it is instruction issue (half the slots busy; a
-// fifth of the instructions are the packed multiply-adds, the others signs,
+// pf 4p4n.  What bounds it is instruction issue (at k = 2 half the slots busy;
+// a sixth of the instructions are the packed multiply-adds, the others signs,
 // weights, stage hand-overs and the adds to y).  pf 4p4n, pn term: 0.46, 0.54,
 // 0.75, 1.46 ms at k = 1, 2, 4, 8; the row kernel's whole product took 1.78
-// and 2.14 ms at k = 1, 2 (0.59 and 0.73 now), the (Z-1)-core kernel takes
-// 0.84 and 1.03 ms at k = 4, 8, so k = 8 stays there.  The price is the multiply-adds with states the neutron core occupies
-// (their x is zero): ((ns - N + 1) / ns)^2 of them are of use, 0.72 at pf 4p4n.
+// and 2.14 ms at k = 1, 2 (0.58 and 0.72 now), the (Z-1)-core kernel takes
+// 0.84 and 1.03 ms at k = 4, 8, so k = 8 stays there.  The price is the
+// multiply-adds with states the neutron core occupies (their x is zero):
+// ((ns - N + 1) / ns)^2 of them are of use, 0.72 at pf 4p4n.
 //
 // One CTA per SM and item: a proton core with all its rows and CP of the K
-// components.  The item's output rows Y live in
-// shared memory.  Four producer warps gather X (cp.async, zeros for occupied
+// components.  The item's output rows Y live in shared memory.  Four producer warps gather X (cp.async, zeros for occupied
 // states) and W into a ring of stages of KC pairs kl; sixteen consumer warps
 // in four groups share it: group g owns the rows of a fixed subset of the
 // proton states i, its warp w the cores 32 w .. 32 w + 31, one core per lane,
