@@ -212,7 +212,8 @@ template <typename T, int K>
 int launch_adj(bs_ctx *c, const T *x, const T *gy, cudaStream_t s, std::vector<int> &cb, std::vector<int> &cl)
 {
     const Device &D = c->dev;
-    adj_pp<T, K><<<D.nrtasks, 128, 0, s>>>(D.rtasks, D.blocks, D.pp_ptr, D.pp_src, x, gy, c->adj_gpp);
+    const AdjPlan::Moves *M = c->adj.have_moves ? c->adj.moves : nullptr;
+    adj_pp<T, K><<<D.nrtasks, 128, 0, s>>>(D.rtasks, D.blocks, M ? M[0].ptr : D.pp_ptr, M ? M[0].src : D.pp_src, x, gy, c->adj_gpp);
     if (!cb.empty()) {
         int *dcb = nullptr, *dcl = nullptr;
         cudaError_t me = cudaMallocAsync((void **)&dcb, cb.size() * sizeof(int), s);
@@ -224,7 +225,8 @@ int launch_adj(bs_ctx *c, const T *x, const T *gy, cudaStream_t s, std::vector<i
         }
         cudaMemcpyAsync(dcb, cb.data(), cb.size() * sizeof(int), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(dcl, cl.data(), cl.size() * sizeof(int), cudaMemcpyHostToDevice, s);
-        adj_nn<T, K><<<(int)cb.size(), 128, 0, s>>>(D.blocks, dcb, dcl, D.nn_ptr, D.nn_src, x, gy, c->adj_gnn);
+        adj_nn<T, K><<<(int)cb.size(), 128, 0, s>>>(D.blocks, dcb, dcl, M ? M[1].ptr : D.nn_ptr, M ? M[1].src : D.nn_src, x, gy,
+                                                           c->adj_gnn);
         cudaFreeAsync(dcb, s);
         cudaFreeAsync(dcl, s);
     }
@@ -914,9 +916,27 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
     const Tables &T = c->tab;
     const Interaction &I = c->inter;
     cudaError_t e;
+    // The products' lists hold no move whose matrix element is zero; its density counts all the same.
     if (!c->adj_gpp) {
-        if ((e = cudaMalloc(&c->adj_gpp, std::max<size_t>(1, T.pp.src.size()) * sizeof(double))) != cudaSuccess ||
-            (e = cudaMalloc(&c->adj_gnn, std::max<size_t>(1, T.nn.src.size()) * sizeof(double))) != cudaSuccess ||
+        bool zeros = false;
+        for (const std::vector<int> &v : I.pairs_by_key)
+            for (int p : v)
+                for (int q : v) zeros = zeros || I.Wpp[(size_t)p * I.npairs + q] == 0.0;
+        for (int spc = 0; zeros && spc < 2; ++spc) {
+            AdjPlan::Moves &m = c->adj.moves[spc];
+            like_moves(c->basis, I, spc, m.list);
+            if ((e = put_plan(c->adj, m.ptr, m.list.ptr)) != cudaSuccess || (e = put_plan(c->adj, m.src, m.list.src)) != cudaSuccess) {
+                (void)cudaGetLastError();
+                c->err = std::string("adjoint: ") + cudaGetErrorString(e);
+                return e == cudaErrorMemoryAllocation ? BS_ENOMEM : BS_ECUDA;
+            }
+        }
+        c->adj.have_moves = zeros;
+    }
+    const LikeJumps &pp = c->adj.have_moves ? c->adj.moves[0].list : T.pp, &nn = c->adj.have_moves ? c->adj.moves[1].list : T.nn;
+    if (!c->adj_gpp) {
+        if ((e = cudaMalloc(&c->adj_gpp, std::max<size_t>(1, pp.src.size()) * sizeof(double))) != cudaSuccess ||
+            (e = cudaMalloc(&c->adj_gnn, std::max<size_t>(1, nn.src.size()) * sizeof(double))) != cudaSuccess ||
             (e = cudaMalloc(&c->adj_rho, std::max<size_t>(1, I.Wpn.size()) * sizeof(double))) != cudaSuccess) {
             c->err = std::string("adjoint: ") + cudaGetErrorString(e);
             (void)cudaGetLastError();
@@ -926,8 +946,8 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
             return BS_ENOMEM;
         }
     }
-    cudaMemsetAsync(c->adj_gpp, 0, std::max<size_t>(1, T.pp.src.size()) * sizeof(double), s);
-    cudaMemsetAsync(c->adj_gnn, 0, std::max<size_t>(1, T.nn.src.size()) * sizeof(double), s);
+    cudaMemsetAsync(c->adj_gpp, 0, std::max<size_t>(1, pp.src.size()) * sizeof(double), s);
+    cudaMemsetAsync(c->adj_gnn, 0, std::max<size_t>(1, nn.src.size()) * sizeof(double), s);
     cudaMemsetAsync(c->adj_rho, 0, std::max<size_t>(1, I.Wpn.size()) * sizeof(double), s);
     // one CTA per (block, neutron column) for the nn densities
     std::vector<int> cb, cl;
@@ -951,7 +971,7 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
         }
     }
     if (rc) return rc;
-    std::vector<double> gpp(T.pp.src.size()), gnn(T.nn.src.size()), rho(I.Wpn.size());
+    std::vector<double> gpp(pp.src.size()), gnn(nn.src.size()), rho(I.Wpn.size());
     cudaMemcpyAsync(gpp.data(), c->adj_gpp, gpp.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
     cudaMemcpyAsync(gnn.data(), c->adj_gnn, gnn.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
     cudaMemcpyAsync(rho.data(), c->adj_rho, rho.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -961,8 +981,8 @@ int run_backward(bs_ctx *c, const void *x, const void *gy, void *gx, double *gth
     }
     const int ns = (int)c->basis.st.size();
     std::vector<double> rho2((size_t)I.npairs * I.npairs, 0.0), rho1p(ns, 0.0), rho1n(ns, 0.0);
-    split_like(c->basis, I, 0, T.pp, gpp, rho2, rho1p);
-    split_like(c->basis, I, 1, T.nn, gnn, rho2, rho1n);
+    split_like(c->basis, I, 0, pp, gpp, rho2, rho1p);
+    split_like(c->basis, I, 1, nn, gnn, rho2, rho1n);
     const int no = (int)c->spe_in.size();
     for (int st = 0; st < ns; ++st) gtheta[c->basis.st[(size_t)st].orb] += rho1p[st] + rho1n[st];
     for (const WTerm &t : c->dWpp) gtheta[no + t.t] += rho2[(size_t)t.at] * t.c;

@@ -381,6 +381,13 @@ struct AdjPlan {
     int nctas = 0, nbatch = 0, nnd = 0;
     int64_t pn_size = 0, pd = 0, nd = 0, nout = 0;
     std::vector<int64_t> like_off, pn_to_w;
+    // the kernels by jumps: lists of all like-particle moves, protons and neutrons, where the products' lists lack some
+    struct Moves {
+        LikeJumps list;
+        int64_t *ptr = nullptr;
+        int32_t *src = nullptr;
+    } moves[2];
+    bool have_moves = false;
     std::vector<void *> owned;
 };
 
@@ -529,6 +536,7 @@ void build_interaction_derivatives(const Basis &B, const Interaction &I, const s
                                    std::vector<WTerm> &pn);
 void release_adj(AdjPlan &P);
 int build_tables(const Basis &B, const Interaction &I, Tables &T, std::string &err, int grid = 152);
+void like_moves(const Basis &B, const Interaction &I, int spc, LikeJumps &L);
 void build_like_lists(const LikeJumps &L, LikeLists &O);
 void build_like_panels(const Basis &B, int spc, int pos, std::vector<LikePanel> &O, int &max_n);
 int like_panel_width(int max_n);

@@ -1110,6 +1110,18 @@ void build_pp_units(const Basis &B, const Interaction &I, Tables &T)
 }
 }  // namespace
 
+// The lists of every two-body move inside a sector, also of those whose matrix element is zero.
+void like_moves(const Basis &B, const Interaction &I, int spc, LikeJumps &L)
+{
+    Interaction all = I;
+    for (const std::vector<int> &v : all.pairs_by_key)
+        for (int p : v)
+            for (int q : v) all.Wpp[(size_t)p * all.npairs + q] = 1.0;
+    LikeCross X;
+    int64_t n = 0;
+    like_jumps(B, all, spc, L, X, n);
+}
+
 int build_tables(const Basis &B, const Interaction &I, Tables &T, std::string &err, int grid)
 {
     (void)err;
